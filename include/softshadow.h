@@ -141,6 +141,11 @@ typedef struct {
     double angular_radius_rad;  /* alpha = r_L > 0                             */
 } ss_sun;
 
+/* ss_shadow_forward takes packets of 32 rays when every
+ * shape field below is left at its default (and SS_FLAG_LANE_LEAVES is not set).
+ * Setting any of block_threads, leaf_level, rays_per_thread, refill_min,
+ * ray_tile_w, strip_len or seed_width selects the single-ray walks, where the
+ * fields left at 0 (-1) take the defaults given with them.  Same results. */
 typedef struct {
     double max_len_m;      /* Lmax: longest ray (m), > 0                       */
     double step_texels;    /* delta / g; 0 selects 0.5                         */

@@ -182,6 +182,13 @@ bool rise_series_ok(const ss_heightfield* hf, const ss_sun* sun, double tmax, in
     return tmax * (4.0 * se / R + 4.0 * tmax / (R * R)) <= 0.03125;
 }
 
+// No launch shape, seeding or leaf size is asked for: the library's own choice.
+bool default_shape(const ss_params* p) {
+    return p->block_threads == 0 && p->leaf_level < 0 && p->rays_per_thread == 0 &&
+           p->refill_min == 0 && p->ray_tile_w == 0 && p->strip_len == 0 && p->seed_width == 0 &&
+           !(p->flags & SS_FLAG_LANE_LEAVES);
+}
+
 enum class FwdKind { Descent, Uniform };
 
 // rays per descent strip when strips are used by default (each ray seeded from
@@ -267,6 +274,15 @@ ss_status shadow_common(FwdKind kind, const ss_heightfield* hf, const float* mip
                    : tasks                ? (stereo ? 22 : 14)
                    : descent              ? 10
                                           : 6;
+    // Packets of rays (ss_packet.cuh) unless a launch shape is asked for: faster than
+    // the walks for every size, mapping, ray set and mode measured, from 1.1x
+    // (2048^2, light-only, sun 0.3 deg: 1.31 -> 1.14 ms) over 2x (4096^2: 16.1 -> 8.0 ms)
+    // to 16x (100 k scattered points: 3.5 -> 0.22 ms); the same within 5 us below
+    // 1,500 rays.  The walks stay for callers that set a shape.
+    if (descent && default_shape(params))
+        a.pk_len = ss::pk_strip_len(rays->mode == SS_RAYS_GRID
+                                        ? ss::pk_grid_strips(hf->nx, hf->ny, 1)
+                                        : (n + 31) / 32);
     cudaError_t e = kind == FwdKind::Descent
                         ? ss::launch_dp_forward(a, block, (cudaStream_t)stream)
                         : ss::launch_uniform_forward(a, block, (cudaStream_t)stream);

@@ -343,6 +343,13 @@ int device_sm_count() {
     return g_sm_count;
 }
 
+// Packets a warp takes one after the other: longer strips seed more of them from
+// the one above, shorter ones fill the GPU and end evenly.
+int32_t pk_strip_len(int64_t packets) {
+    const int64_t len = packets / ((int64_t)device_sm_count() * 32 * 4);
+    return (int32_t)(len < 1 ? 1 : len > kPkMaxLen ? kPkMaxLen : len);
+}
+
 // Grid-stride kernels: one wave of resident blocks (occupancy x SMs), fewer
 // when there is not enough work.
 template <typename K>

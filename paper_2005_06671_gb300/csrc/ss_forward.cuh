@@ -509,12 +509,17 @@ inline bool use_task_descent(const FwdArgs& a, bool grid, bool stereo, bool ligh
            a.kleaf <= (grid && !stereo ? 1 : 2) && !(a.flags & 0x10u);   // SS_FLAG_LANE_LEAVES
 }
 
+// defined in ss_packet.cuh
+template <bool C, bool G, bool P, bool L, bool S>
+static void launch_packet(const FwdArgs& a, cudaStream_t s);
+
 template <bool C, bool G, bool P, bool L, bool S>
 struct DpLaunch {
     static cudaError_t go(const FwdArgs& a, int grid, int block, cudaStream_t s) {
-        bool tasks = false;
+        bool tasks = a.pk_len > 0;
+        if (tasks) launch_packet<C, G, P, L, S>(a, s);
         if constexpr (!L) {
-            if (use_task_descent(a, G, S, L)) {
+            if (!tasks && use_task_descent(a, G, S, L)) {
                 dp_task_kernel<C, G, P, S><<<grid, block, 0, s>>>(a);
                 tasks = true;
             }

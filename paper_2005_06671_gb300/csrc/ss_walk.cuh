@@ -381,10 +381,14 @@ __device__ __forceinline__ float seed_geo(const Tile& T, const RayF& rf, int32_t
 // ahead (0.5-texel steps), so a window around j_src alone would miss it.
 // (Grid rays.  Listed rays keep the window at j_src: on the polar view the
 // centring saved 5% of the probes but measured 4% slower.)
-__device__ __forceinline__ int32_t seed_centre(const RayF& rf, int32_t j_src, float du, float dv) {
-    const float a2 = rf.au * rf.au + rf.av * rf.av;
-    const float sh = a2 > 0.0f ? __fdividef(du * rf.au + dv * rf.av, a2) : 0.0f;
+__device__ __forceinline__ int32_t seed_centre_of(float au, float av, int32_t j_src, float du,
+                                                  float dv) {
+    const float a2 = au * au + av * av;
+    const float sh = a2 > 0.0f ? __fdividef(du * au + dv * av, a2) : 0.0f;
     return j_src + (int32_t)rintf(fminf(fmaxf(sh, -1.0e6f), 1.0e6f));
+}
+__device__ __forceinline__ int32_t seed_centre(const RayF& rf, int32_t j_src, float du, float dv) {
+    return seed_centre_of(rf.au, rf.av, j_src, du, dv);
 }
 
 // Seed of a newly drawn ray: with a finished neighbour (`near`), its samples
