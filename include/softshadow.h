@@ -141,7 +141,7 @@ typedef struct {
     double angular_radius_rad;  /* alpha = r_L > 0                             */
 } ss_sun;
 
-/* ss_shadow_forward takes packets of 32 rays when every
+/* The descent (ss_shadow_forward, the batch) takes packets of 32 rays when every
  * shape field below is left at its default (and SS_FLAG_LANE_LEAVES is not set).
  * Setting any of block_threads, leaf_level, rays_per_thread, refill_min,
  * ray_tile_w, strip_len or seed_width selects the single-ray walks, where the
@@ -321,8 +321,9 @@ ss_status ss_shadow_backward_ws(const ss_heightfield* hf, const ss_rays* rays, c
  * counterpart in the paper is drawing many visible tiles per frame (Sec. 3.3,
  * virtual texturing; Sec. 6.3).  Grid-mode rays (one per texel centre),
  * gnomonic tiles.  params (max_len_m, step_texels, ...) apply to every item;
- * zero shape fields take the batch defaults: exact walks in 64 x 64 chunks of
- * texels (rays_per_thread 128, ray_tile_w 64) with column seeds and services
+ * default shape fields select packets of 32 rays, strips of which are the queue's
+ * chunks; with a shape field set the rest take the walks' batch defaults: exact
+ * walks in 64 x 64 chunks of texels (rays_per_thread 128, ray_tile_w 64) with column seeds and services
  * at 14 idle lanes, light-only walks in runs of 512 (rays_per_thread 16) with
  * services at 6.  A caller who sets rays_per_thread sets ray_tile_w too
  * (0 = runs of consecutive texels). */

@@ -328,6 +328,8 @@ ss_status batch_prepare(const ss_batch_item* items, int32_t n, const ss_params* 
     auto* prefix = reinterpret_cast<int64_t*>(B.image.data() + desc_bytes);
     B.layouts.resize(n);
     prefix[0] = 0;
+    int32_t n_poly = 0;
+    int64_t n_packets = 0;
     for (int32_t i = 0; i < n; ++i) {
         const ss_batch_item& it = items[i];
         ss_status st = check_tile(&it.hf, 2);
@@ -357,8 +359,18 @@ ss_status batch_prepare(const ss_batch_item* items, int32_t n, const ss_params* 
         d.n_rays = (int64_t)it.hf.nx * it.hf.ny;
         d.poly = rise_series_ok(&it.hf, &it.sun, J * delta, SS_RAYS_GRID) ? 1 : 0;
         d.tile_w = tile_w;
-        prefix[i + 1] = prefix[i] + ss::chunk_count(d.n_rays, it.hf.nx, it.hf.ny, chunk, tile_w);
+        n_poly += d.poly;
+        n_packets += ss::pk_grid_strips(it.hf.nx, it.hf.ny, 1);
     }
+    // packets of rays (batch_packet.cu) unless a launch shape is asked for; one
+    // form of the rise serves a launch, so a batch that mixes both takes chunks
+    const int32_t pk_len = default_shape(params) && (n_poly == 0 || n_poly == n)
+                               ? ss::pk_strip_len(n_packets) : 0;
+    for (int32_t i = 0; i < n; ++i)
+        prefix[i + 1] = prefix[i] +
+                        (pk_len > 0 ? ss::pk_grid_strips(descs[i].T.nx, descs[i].T.ny, pk_len)
+                                    : ss::chunk_count(descs[i].n_rays, descs[i].T.nx,
+                                                      descs[i].T.ny, chunk, tile_w));
     unsigned long long* counter;
     ss::BatchItemDesc* ditems;
     int64_t* dprefix;
@@ -376,6 +388,8 @@ ss_status batch_prepare(const ss_batch_item* items, int32_t n, const ss_params* 
                                          : (B.args.light_only ? 1 : kDefaultStrip);
     B.args.colseed = (params->strip_len == 0 && !B.args.light_only && tile_w > 0) ? 1 : 0;
     B.args.seed_w = params->seed_width > 0 ? params->seed_width : 1;   // grid rays
+    B.args.pk_len = pk_len;
+    B.args.poly = n_poly == n ? 1 : 0;
     B.args.lane_leaves = (params->flags & SS_FLAG_LANE_LEAVES) ? 1 : 0;
     return SS_OK;
 }

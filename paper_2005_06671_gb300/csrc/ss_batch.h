@@ -37,6 +37,8 @@ struct BatchArgs {
     int32_t colseed;                // rectangular chunks: single rays, column seeds
     int32_t seed_w;                 // half-width of a seed window
     int32_t lane_leaves;            // SS_FLAG_LANE_LEAVES: leaves in the walking lane
+    int32_t pk_len;                 // > 0: packets of rays, chunks are strips of so many
+    int32_t poly;                   // packets: the rise series is valid for every ray
 };
 
 constexpr int32_t kBatchSeedW = 64;    // widest chunk with a column-seed table
@@ -47,6 +49,7 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 size_t batch_workspace_bytes(int32_t n_items);
 void batch_layout(void* ws, int32_t n_items, unsigned long long** counter, BatchItemDesc** items,
                   int64_t** prefix);
+cudaError_t launch_batch_packets(const BatchArgs& a, bool count, cudaStream_t s);
 cudaError_t launch_batch_forward(const BatchArgs& a, int block, bool count, cudaStream_t s);
 
 }  // namespace ss

@@ -1,4 +1,4 @@
-"""The packet descent (the default ss_shadow_forward) against uniform
+"""The packet descent (the default ss_shadow_forward and batch) against uniform
 stepping, which evaluates every sample with the same arithmetic: argmin, cost and
 light have to be the same bits whatever the shape, mapping, sun or ray set.  In
 light-only mode the light is, and the argmin of rays in the penumbra."""
@@ -90,3 +90,22 @@ def test_nan_heights(proj):
     ok = torch.isfinite(hf.h).reshape(-1)     # (rays on a NaN texel are unspecified)
     assert torch.equal(a["argmin"][ok], b["argmin"][ok])
     assert torch.equal(a["light"][ok], b["light"][ok])
+
+
+@pytest.mark.parametrize("elev", [1.0, 35.0])
+@pytest.mark.parametrize("light_only", [False, True])
+def test_batch(elev, light_only):
+    ss = _ss()
+    hfs = [_tile(nx, ny, 20.0, pad=p, seed=k)
+           for k, (nx, ny, p) in enumerate([(2, 2, 0), (65, 33, 1), (128, 96, 0), (7, 300, 2)])]
+    suns = [ss.Sun(math.radians(elev + 0.1 * k), 0.9 * k) for k in range(4)]
+    b = ss.Batch(hfs, suns, 20e3, want_cost=True, light_only=light_only)
+    for go in (b.submit, b.launch):
+        for hf, sun, o in zip(hfs, suns, go()):
+            r = ss.ss_shadow_uniform(hf, ss.ss_build_maxmip(hf), sun, 20e3, early_exit=False)
+            assert torch.equal(o["light"], r["light"])
+            pen = (r["light"] > 0) & (r["light"] < 1) if light_only else slice(None)
+            assert torch.equal(o["argmin"][pen], r["argmin"][pen])
+            assert torch.equal(o["cost"][pen], r["cost"][pen])
+            o["light"].fill_(7.0)
+    b.close()
