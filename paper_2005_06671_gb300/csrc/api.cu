@@ -189,6 +189,14 @@ bool default_shape(const ss_params* p) {
            !(p->flags & SS_FLAG_LANE_LEAVES);
 }
 
+// Packets of rays (ss_packet.cuh, batch_packet.cu): the default shape, and rays short
+// enough in texels for the float32 floors of ss_leaf2.cuh (2^22, reached only by
+// rays of a few hundred thousand texels from origins far off the tile).
+bool takes_packets(const ss_params* p, int32_t J) {
+    const double st = p->step_texels == 0.0 ? 0.5 : p->step_texels;
+    return default_shape(p) && (double)J * st <= 2.5e5;
+}
+
 enum class FwdKind { Descent, Uniform };
 
 // rays per descent strip when strips are used by default (each ray seeded from
@@ -275,14 +283,15 @@ ss_status shadow_common(FwdKind kind, const ss_heightfield* hf, const float* mip
                    : descent              ? 10
                                           : 6;
     // Packets of rays (ss_packet.cuh) unless a launch shape is asked for: faster than
-    // the walks for every size, mapping, ray set and mode measured, from 1.1x
-    // (2048^2, light-only, sun 0.3 deg: 1.31 -> 1.14 ms) over 2x (4096^2: 16.1 -> 8.0 ms)
-    // to 16x (100 k scattered points: 3.5 -> 0.22 ms); the same within 5 us below
+    // the walks for every size, mapping, ray set and mode measured, from 1.2x
+    // (2048^2, light-only, sun 0.3 deg: 1.31 -> 1.06 ms) over 2.2x (4096^2: 15.9 -> 7.1 ms)
+    // to 15x (100 k scattered points: 3.3 -> 0.22 ms); the same within 5 us below
     // 1,500 rays.  The walks stay for callers that set a shape.
-    if (descent && default_shape(params))
+    if (descent && takes_packets(params, J))
         a.pk_len = ss::pk_strip_len(rays->mode == SS_RAYS_GRID
                                         ? ss::pk_grid_strips(hf->nx, hf->ny, 1)
-                                        : (n + 31) / 32);
+                                        : (n + 31) / 32,
+                                    light_only);
     cudaError_t e = kind == FwdKind::Descent
                         ? ss::launch_dp_forward(a, block, (cudaStream_t)stream)
                         : ss::launch_uniform_forward(a, block, (cudaStream_t)stream);
@@ -330,6 +339,7 @@ ss_status batch_prepare(const ss_batch_item* items, int32_t n, const ss_params* 
     prefix[0] = 0;
     int32_t n_poly = 0;
     int64_t n_packets = 0;
+    bool packets = true;
     for (int32_t i = 0; i < n; ++i) {
         const ss_batch_item& it = items[i];
         ss_status st = check_tile(&it.hf, 2);
@@ -360,12 +370,13 @@ ss_status batch_prepare(const ss_batch_item* items, int32_t n, const ss_params* 
         d.poly = rise_series_ok(&it.hf, &it.sun, J * delta, SS_RAYS_GRID) ? 1 : 0;
         d.tile_w = tile_w;
         n_poly += d.poly;
+        packets = packets && takes_packets(params, J);
         n_packets += ss::pk_grid_strips(it.hf.nx, it.hf.ny, 1);
     }
     // packets of rays (batch_packet.cu) unless a launch shape is asked for; one
     // form of the rise serves a launch, so a batch that mixes both takes chunks
-    const int32_t pk_len = default_shape(params) && (n_poly == 0 || n_poly == n)
-                               ? ss::pk_strip_len(n_packets) : 0;
+    const int32_t pk_len = packets && (n_poly == 0 || n_poly == n)
+                               ? ss::pk_strip_len(n_packets, batch_light) : 0;
     for (int32_t i = 0; i < n; ++i)
         prefix[i + 1] = prefix[i] +
                         (pk_len > 0 ? ss::pk_grid_strips(descs[i].T.nx, descs[i].T.ny, pk_len)

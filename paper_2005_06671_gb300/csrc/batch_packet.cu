@@ -9,7 +9,7 @@
 // re-evaluated in FP64 by a second kernel over the same strips, with full warps.
 //
 // Bound by instruction issue, as ss_packet.cuh.  16 tiles of 512^2 to 4096^2 (67 M
-// rays, a sun each) take 36.3 ms against 87.5 ms with batch_task_kernel; 16 tiles of
+// rays, a sun each) take 33.6 ms against 89.9 ms with batch_task_kernel; 16 tiles of
 // 512^2 1.69 against 11.7 ms, 4 tiles of 256^2 0.17 against 7.3 ms (its chunks of
 // 4,096 texels leave most of the GPU's warps without one).
 #include "ss_batch.h"
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kPkThreads, SS_PK_MIN_BLOCKS) batch_packet_ker
 // FP64 re-evaluation of the rays left pending (refine_kernel over the strips): a
 // block gathers the pending rays of kBatchRefineStrips strips, then every thread
 // takes one.
-constexpr int kBatchRefineStrips = 8;
+constexpr int kBatchRefineStrips = 4;
 
 __global__ void __launch_bounds__(256) batch_refine_kernel(const BatchArgs a) {
     __shared__ int64_t s_ray[kBatchRefineStrips * kPkMaxLen * kPkRows * kPkCols];

@@ -49,8 +49,8 @@ inline int64_t pk_grid_strips(int32_t nx, int32_t ny, int32_t len) {
     return (int64_t)((nx + kPkCols - 1) / kPkCols) *
            ((ny + (int64_t)kPkRows * len - 1) / ((int64_t)kPkRows * len));
 }
-constexpr int kPkMaxLen = 8;
-int32_t pk_strip_len(int64_t packets);
+constexpr int kPkMaxLen = 16;
+int32_t pk_strip_len(int64_t packets, bool light);
 
 struct BwdArgs {
     Tile T;

@@ -29,15 +29,21 @@
 // Listed rays need not be neighbours, so their blocks are tasks from the whole
 // ray down (pk_descend_list); the rest is the same.
 //
-// What bounds it: instruction issue (72% of slots at 2048^2, 30.4 of 32 lanes
-// active; the ALU pipe 54% busy, DRAM 0.1%).  Measured (GB300, mipmap included): 4096^2
-// 16.1 -> 8.0 ms against the task descent of ss_task.cuh, 1531 x 1021 2.75 -> 0.85 ms,
-// 256^2 1.12 -> 0.086 ms, 1200 x 1000 stereographic 3.9 -> 0.95 ms, 1.04 M view
-// points 13.2 -> 2.4 ms, 100 k scattered points 3.5 -> 0.22 ms (the task descent's
+// What bounds it: instruction issue (76% of slots at 2048^2, 30 of 32 lanes active,
+// the ALU pipe 51% busy, shared and L1 wavefronts 63%, DRAM 0.1%); per packet of 32
+// rays 11.4 k instructions: 12 leaf passes 3.8 k, 13 node passes ~3 k, tests 1 k,
+// setup 0.6 k, unions 0.4 k.  Measured (GB300, pass with the mipmap) against the task
+// descent of ss_task.cuh: 4096^2 15.9 -> 7.1 ms, 1531 x 1021 2.71 -> 0.74 ms, 256^2
+// 1.15 -> 0.076 ms, 1200 x 1000 stereographic 3.83 -> 0.87 ms, 1.04 M view points
+// 13.2 -> 2.4 ms, 100 k scattered points 3.5 -> 0.21 ms (the task descent's
 // blocks of 6,144 or 3,072 rays leave most SMs idle on all but the first).
+// Scalar leaves, tests and one push per node of the packet took 8.0 ms at 4096^2;
+// tasks of 16 samples bounded in quarters 7.0, but light-only passes 9% and view
+// points 16% more.
 #pragma once
 
 #include "ss_forward.cuh"
+#include "ss_leaf2.cuh"
 #include "ss_leaftask.cuh"
 
 namespace ss {
@@ -53,11 +59,11 @@ constexpr int kPkNodeRing = 64;    // < 32 tasks wait when up to 32 are added
 constexpr int kPkStackFull = 128, kPkStack = 384;
 static_assert(kPkStackFull + 32 + 15 * 13 <= kPkStack, "stack of block tasks");
 constexpr int kPkLeafRing = 128;   // < 32 wait when up to 64 are added
-constexpr uint32_t kPkSparse = 0x80000000u;   // leaf task of samples j, 2j, 4j, 8j
+constexpr uint32_t kPkSparse = 0x80000000u;   // leaf task of samples j, 6j, 11j, 16j
 constexpr float kPkSpread = 512.0f;   // listed rays: neighbours' minima serve as seeds
 // Blocks of 4 warps (nothing is shared between warps but the level table; 2 warps
-// measure the same), 8 of them per SM: 64 registers.  Three suns at 4096^2: 23.5 ms
-// with 8, 23.7 with 6, 23.0 with 10 (48 registers, spills on other instances).
+// measure the same), 8 of them per SM: 64 registers.  Three suns at 4096^2: 20.2 ms
+// with 8, 20.9 with 6.
 #ifndef SS_PK_MIN_BLOCKS
 #define SS_PK_MIN_BLOCKS 8
 #endif
@@ -170,12 +176,11 @@ __device__ __forceinline__ void pk_load(const Warp& W, int slot, RayF& r, int32_
 // it), as <= 2x2 cells of the coarsest level whose cells cover it.
 __device__ __forceinline__ float pk_box_max(const Tile& T, const LevelTab& L, int32_t levels,
                                             float xlo, float xhi, float ylo, float yhi) {
-    const int32_t x0 = max(__float2int_rd(xlo), 0);
-    const int32_t x1 = min(__float2int_rd(xhi), T.nx - 2) + 1;
-    const int32_t y0 = max(__float2int_rd(ylo), 0);
-    const int32_t y1 = min(__float2int_rd(yhi), T.ny - 2) + 1;
-    // (a box off the tile is empty of samples: any cell of the tile will do)
-    const int32_t ax = min(x0, T.nx - 1), bx = max(x1, ax), ay = min(y0, T.ny - 1), by = max(y1, ay);
+    // (clamped so that a box off the tile reads cells of the tile's border)
+    const int32_t ax = __vimin_s32_relu(__float2int_rd(xlo), T.nx - 1);
+    const int32_t bx = __vimin_s32_relu(__float2int_rd(xhi), T.nx - 2) + 1;
+    const int32_t ay = __vimin_s32_relu(__float2int_rd(ylo), T.ny - 1);
+    const int32_t by = __vimin_s32_relu(__float2int_rd(yhi), T.ny - 2) + 1;
     const int32_t ext = max(bx - ax, by - ay);
     int32_t m = ext <= 1 ? 0 : 31 - __clz(ext);
     m += (((bx >> m) - (ax >> m)) > 1 || ((by >> m) - (ay >> m)) > 1) ? 1 : 0;
@@ -286,22 +291,29 @@ __device__ __forceinline__ void pk_leaf_pass(const Tile& T, Warp& W, PkRings& Q,
         RayF q;
         int32_t jl, jh;
         pk_load(W, slot, q, jl, jh);
-        float best = INFINITY;
-        int32_t bj = 0;
+        const int32_t d = sparse ? 5 * j0 : 1;
+        int32_t j[4];
+        float c[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int32_t j = min(max(sparse ? j0 << i : j0 + i, jl), jh);
-            float rise;
-            const float c = leaf_cost<kGrid, kPoly, kStereo>(T, q, j, rise);
-            if (c < best) {   // (ascending j: the smallest index on ties)
-                best = c;
-                bj = j;
+            j[i] = min(j0 + i * d, jh);
+            if (!kGrid) j[i] = max(j[i], jl);   // (a grid ray's first usable sample is 1)
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) {
+            if constexpr (kPoly) {
+                leaf_cost2<kGrid, kStereo>(T, q, j[i], j[i + 1], c[i], c[i + 1]);
+            } else {
+                float rise;
+                c[i] = leaf_cost<kGrid, kPoly, kStereo>(T, q, j[i], rise);
+                c[i + 1] = leaf_cost<kGrid, kPoly, kStereo>(T, q, j[i + 1], rise);
             }
         }
-        if (best < INFINITY) {
-            const unsigned long long key = pack_key(best, bj);
-            // (a stale key is only larger: no better minimum is lost)
-            if (key < W.key[slot]) atomicMin(&W.key[slot], key);
+        const float best = fminf(fminf(c[0], c[1]), fminf(c[2], c[3]));   // (NaN costs drop out)
+        // (a stale key is only larger: no better minimum is lost)
+        if (best < INFINITY && best <= key_cost(W.key[slot])) {
+            const int32_t bj = c[0] == best ? j[0] : c[1] == best ? j[1] : c[2] == best ? j[2] : j[3];
+            atomicMin(&W.key[slot], pack_key(best, bj));
         }
         if (kCount) atomicAdd(&W.cnt[1][slot], 4);
     }
@@ -353,8 +365,8 @@ __device__ __forceinline__ void pk_node_pass(const Tile& T, const LevelTab& L, i
         const float hg = __fmaf_rn(-0.2503f * q.y * dt, dt, q.w);
         const float f0 = pk_f(q.y, p, hg, t0), f1 = pk_f(q.y, p, hg, t1);
         const float f2 = pk_f(q.y, p, hg, t2);
-        pa = !(fminf(f0, f1) > Ma) && s + 1 <= jh && s + half >= jl;
-        pb = !(fminf(f1, f2) > Mb) && s + half + 1 <= jh && s + 2 * half >= jl;
+        pa = !(fminf(f0, f1) > Ma) && s + 1 <= jh && (kGrid || s + half >= jl);
+        pb = !(fminf(f1, f2) > Mb) && s + half + 1 <= jh && (kGrid || s + 2 * half >= jl);
         if (kCount) atomicAdd(&W.cnt[0][slot], 2);
     }
     if (kGrid) Q.nh = (Q.nh + n) & (kPkNodeRing - 1);
@@ -407,7 +419,7 @@ __device__ __forceinline__ void pk_descend(const Tile& T, const LevelTab& L, int
     const int32_t jmax = __reduce_max_sync(kFull, jh);
     int32_t s = 0, sn = 0;              // next batch of top blocks; the current top block
     uint32_t tops = 0, any = 0;         // the lane's / the packet's top blocks left
-    uint32_t nodes = 0, un = 0;         // likewise of the current top block's nodes
+    uint32_t nodes = 0, un = 0;         // nodes left of the current top block / lanes with some
     int32_t st = 0;                     // first sample of the current batch of top blocks
     bool flush = true;                  // drain the rings (first: the seeds)
     while (true) {
@@ -419,10 +431,11 @@ __device__ __forceinline__ void pk_descend(const Tile& T, const LevelTab& L, int
             pk_node_pass<kCount, true, kPoly, kLight, kStereo>(T, L, levels, W, Q, lane);
             continue;
         }
-        if (un) {                       // a node's surviving rays become tasks
-            const int n = __ffs(un) - 1;
-            un &= un - 1u;
-            pk_push_nodes(W, Q, (nodes >> n) & 1u, (sn >> kPkNodeLog) + n, lane);
+        if (un) {                       // each lane's next surviving node becomes a task
+            const int n = __ffs(nodes) - 1;
+            pk_push_nodes(W, Q, nodes != 0u, (sn >> kPkNodeLog) + n, lane);
+            nodes &= nodes - 1u;
+            un = __ballot_sync(kFull, nodes != 0u);
             continue;
         }
         flush = false;
@@ -462,29 +475,31 @@ __device__ __forceinline__ void pk_descend(const Tile& T, const LevelTab& L, int
         const int32_t nv = nodes && jh > base ? min((jh - base + (1 << log) - 1) >> log, 32) : 0;
         const int32_t ng = min((jmax - base + (1 << log) - 1) >> log, 32);   // of any ray's
         const float tb = (float)base * d;
+        const F2 c2 = f2(q.c), p2 = f2(p), hg2 = f2(hg), dt2 = f2(dt);
         float f0 = pk_f(q.c, p, hg, tb);
 #pragma unroll 2
         for (int g = 0; g < ng; g += 4) {
             const float4 M4 = *reinterpret_cast<const float4*>(&W.M[g]);
-            const float tg = __fmaf_rn((float)g, dt, tb);
-            const float f1 = pk_f(q.c, p, hg, tg + dt), f2 = pk_f(q.c, p, hg, __fmaf_rn(2.0f, dt, tg));
-            const float f3 = pk_f(q.c, p, hg, __fmaf_rn(3.0f, dt, tg));
-            const float f4 = pk_f(q.c, p, hg, __fmaf_rn(4.0f, dt, tg));
+            const F2 tg = f2(__fmaf_rn((float)g, dt, tb));
+            const F2 ta = f2_fma(f2(1.0f, 2.0f), dt2, tg), tc = f2_fma(f2(3.0f, 4.0f), dt2, tg);
+            float f1, f2v, f3, f4;
+            f2_get(f2_fma(f2_fma(c2, ta, p2), ta, hg2), f1, f2v);
+            f2_get(f2_fma(f2_fma(c2, tc, p2), tc, hg2), f3, f4);
             uint32_t b = !(fminf(f0, f1) > M4.x) ? 1u : 0u;
-            b |= !(fminf(f1, f2) > M4.y) ? 2u : 0u;
-            b |= !(fminf(f2, f3) > M4.z) ? 4u : 0u;
+            b |= !(fminf(f1, f2v) > M4.y) ? 2u : 0u;
+            b |= !(fminf(f2v, f3) > M4.z) ? 4u : 0u;
             b |= !(fminf(f3, f4) > M4.w) ? 8u : 0u;
             mask |= b << g;
             f0 = f4;
         }
         mask &= nv >= 32 ? kFull : (1u << nv) - 1u;
-        const uint32_t all = __reduce_or_sync(kFull, mask);
         if (log == kPkNodeLog) {
             nodes = mask;
-            un = all;
+            un = __ballot_sync(kFull, mask != 0u);
         } else {
             tops = mask;
-            any = all;
+            any = __reduce_or_sync(kFull, mask);
+            nodes = 0;
         }
         __syncwarp();                   // W.M is reused by the next batch
     }
@@ -534,8 +549,15 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
         v0 = rf.v0;
         au = rf.au;
         av = rf.av;
-        pk_range(rf.u0, U.u0);
-        pk_range(rf.v0, U.v0);
+        if constexpr (kGrid) {   // (8 x 4 texels, the last lane's the far corner)
+            U.u0[0] = __shfl_sync(kFull, rf.u0, 0);
+            U.v0[0] = __shfl_sync(kFull, rf.v0, 0);
+            U.u0[1] = __shfl_sync(kFull, rf.u0, 31);
+            U.v0[1] = __shfl_sync(kFull, rf.v0, 31);
+        } else {
+            pk_range(rf.u0, U.u0);
+            pk_range(rf.v0, U.v0);
+        }
         if constexpr (kGrid) {
             pk_range(rf.au, U.au);
             pk_range(rf.av, U.av);
@@ -557,7 +579,7 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
     if (kCount) W.cnt[0][lane] = W.cnt[1][lane] = 0;
     PkRings Q = { 0, 0, 0, 0 };
     // seeds: samples around where the neighbour's argmin lies along this ray, else
-    // samples 1, 2, 4, ... 2^15 (at most 4 tasks per lane: the ring holds them)
+    // samples 1, 6, 11, 16, 96, ... 2^16 (at most 4 tasks per lane: the ring holds them)
     const bool close =
         kGrid || fmaxf(U.u0[1] - U.u0[0], U.v0[1] - U.v0[0]) <= kPkSpread;   // neighbours
     const bool near = jh > 0 && jc >= 0 && close;
