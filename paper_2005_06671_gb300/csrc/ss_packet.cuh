@@ -35,7 +35,7 @@
 // setup 0.6 k, unions 0.4 k.  Measured (GB300, pass with the mipmap) against the task
 // descent of ss_task.cuh: 4096^2 15.9 -> 7.1 ms, 1531 x 1021 2.71 -> 0.74 ms, 256^2
 // 1.15 -> 0.076 ms, 1200 x 1000 stereographic 3.83 -> 0.87 ms, 1.04 M view points
-// 13.2 -> 2.4 ms, 100 k scattered points 3.5 -> 0.21 ms (the task descent's
+// 13.2 -> 1.9 ms, 100 k scattered points 3.5 -> 0.21 ms (the task descent's
 // blocks of 6,144 or 3,072 rays leave most SMs idle on all but the first).
 // Scalar leaves, tests and one push per node of the packet took 8.0 ms at 4096^2;
 // tasks of 16 samples bounded in quarters 7.0, but light-only passes 9% and view
@@ -580,43 +580,50 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
     PkRings Q = { 0, 0, 0, 0 };
     // seeds: samples around where the neighbour's argmin lies along this ray, else
     // samples 1, 6, 11, 16, 96, ... 2^16 (at most 4 tasks per lane: the ring holds them)
-    const bool close =
-        kGrid || fmaxf(U.u0[1] - U.u0[0], U.v0[1] - U.v0[0]) <= kPkSpread;   // neighbours
-    const bool near = jh > 0 && jc >= 0 && close;
-    const unsigned mn = __ballot_sync(kFull, near);
-    if (near)
-        W.leaf[__popc(mn & lanemask_lt())] = ((uint32_t)min(max(jc - 1, 1), jh) << 5) | (uint32_t)lane;
-    Q.lc = __popc(mn);
-    const bool sparse = !kLight && jh > 0 && !near;
-    for (int32_t j = 1; j <= 4096; j <<= 4) {
-        const bool mine = sparse && j <= jh;
-        const unsigned mj = __ballot_sync(kFull, mine);
+    const auto push_seed = [&](bool mine, uint32_t first) {
+        const unsigned m = __ballot_sync(kFull, mine);
         if (mine)
-            W.leaf[Q.lc + __popc(mj & lanemask_lt())] = kPkSparse | ((uint32_t)j << 5) | (uint32_t)lane;
-        Q.lc += __popc(mj);
-    }
-    __syncwarp();
+            W.leaf[(Q.lh + Q.lc + __popc(m & lanemask_lt())) & (kPkLeafRing - 1)] =
+                (first << 5) | (uint32_t)lane;
+        Q.lc += __popc(m);
+    };
+    const auto near_seed = [&](bool mine, int32_t j) {
+        push_seed(mine && j >= 0, (uint32_t)min(max(j - 1, 1), max(jh, 1)));
+    };
+    const auto sparse_seeds = [&](bool mine) {
+        for (int32_t j = 1; j <= 4096; j <<= 4)
+            push_seed(mine && j <= jh, (kPkSparse >> 5) | (uint32_t)j);
+    };
     if constexpr (kGrid) {
+        near_seed(jh > 0, jc);
+        sparse_seeds(!kLight && jh > 0 && jc < 0);
+        __syncwarp();
         pk_descend<kCount, kPoly, kLight, kStereo>(T, L, levels, W, U, q, jh, csat, Q, lane);
     } else {
-        // listed rays: the seeds, then around where the other rays' minima lie
-        int d = kLight || !close ? 0 : 16;
-        while (true) {
-            while (Q.lc > 0) pk_leaf_pass<kCount, kGrid, kPoly, kStereo>(T, W, Q, lane);
-            if (d == 0) break;
-            const int32_t jo = key_j(W.key[lane ^ d]);
-            const float4 o = W.ray[3][lane ^ d];
-            const int32_t jn = jo > 0 ? seed_centre_of(au, av, jo, o.y - u0, o.z - v0) : 0;
-            const bool mine = jh > 0 && jn > 0;
-            const unsigned m = __ballot_sync(kFull, mine);
-            if (mine)
-                W.leaf[(Q.lh + __popc(m & lanemask_lt())) & (kPkLeafRing - 1)] =
-                    ((uint32_t)min(max(jn - 1, 1), jh) << 5) | (uint32_t)lane;
-            Q.lc = __popc(m);
-            __syncwarp();
-            d >>= 1;
+        // Listed rays that are neighbours (a view's): every fourth ray first, seeded as
+        // above and around each other's minima, then the others around the minima of
+        // the two nearest of those.
+        const bool close = fmaxf(U.u0[1] - U.u0[0], U.v0[1] - U.v0[0]) <= kPkSpread;
+        const bool two = close && !kLight;
+        for (int phase = 0; phase < (two ? 2 : 1); ++phase) {
+            const bool go = jh > 0 && (!two || ((lane & 3) == 0) == (phase == 0));
+            const int rounds = !two ? 1 : phase == 0 ? 4 : 2;
+            for (int r = 0; r < rounds; ++r) {
+                if (r == 0 && phase == 0) {
+                    near_seed(go && close, jc);
+                    sparse_seeds(!kLight && go && !(close && jc >= 0));
+                } else {
+                    const int src = phase == 0 ? lane ^ (32 >> r)
+                                    : r == 0 ? lane & 28 : (lane & 28) + (lane < 28 ? 4 : -4);
+                    const int32_t jo = key_j(W.key[src]);
+                    const float4 o = W.ray[3][src];
+                    near_seed(go && jo > 0, seed_centre_of(au, av, jo, o.y - u0, o.z - v0));
+                }
+                __syncwarp();
+                while (Q.lc > 0) pk_leaf_pass<kCount, kGrid, kPoly, kStereo>(T, W, Q, lane);
+            }
+            pk_descend_list<kCount, kPoly, kLight, kStereo>(T, L, levels, W, go ? jh : 0, Q, lane);
         }
-        pk_descend_list<kCount, kPoly, kLight, kStereo>(T, L, levels, W, jh, Q, lane);
     }
     const unsigned long long key = W.key[lane];
     const int32_t bj = kLight && key_j(key) == 0 ? -1 : key_j(key);
