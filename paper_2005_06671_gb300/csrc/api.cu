@@ -150,7 +150,7 @@ ss::Tile make_tile(const ss_heightfield* hf, const ss_sun* sun, int32_t J, doubl
     split(s[0], sx_hi, T.sx_lo);
     split(s[1], sy_hi, T.sy_lo);
     split(2.0 * R / g, T.k2_hi, T.k2_lo);
-    T.szR_f = (float)(s[2] / R);
+    split(s[2] / R, T.szR_f, T.szR_lo);
     return T;
 }
 

@@ -59,7 +59,7 @@ struct Tile {
     float g_f, cx_f, cy_f;     // (float)g, (float)cx, (float)cy (converted once, on the host)
     // float-float (hi + lo) copies for the grid-ray setup (df_* below)
     float g_hi, g_lo, R_lo, RR_hi, RR_lo, delta_hi, delta_lo, igR_hi, igR_lo;
-    float Rsx_hi, Rsx_lo, Rsy_hi, Rsy_lo, sz_lo, szR_f;
+    float Rsx_hi, Rsx_lo, Rsy_hi, Rsy_lo, sz_lo, szR_f, szR_lo;
     // and for the stereographic setup: sx, sy (low words), 2R/g
     float sx_lo, sy_lo, k2_hi, k2_lo;
 };
@@ -452,12 +452,18 @@ __device__ __forceinline__ DF df_div(DF x, DF y) {
 
 __device__ __forceinline__ double df_to_double(DF x) { return (double)x.hi + (double)x.lo; }
 
+// The local frame of a ray in float-float (the fields of Geom64; b: gnomonic, Bu, Bv,
+// ia0: stereographic).
+struct GeomDF {
+    DF rho, irho, se, Au, Av, b, Bu, Bv, ia0;
+    DF n[3];
+};
+
 // geom64_stereo's fields from float-float arithmetic (relative error ~1e-13
 // against its ~1e-16): the divisions, the square root and the products run on
-// the float32 pipes, and the FP64 values are assembled from the two words.
-// (u, v): origin texel coordinates (float); hp: origin height.
-__device__ __forceinline__ void geom_stereo_df(const Tile& T, float uf, float vf, DF hp,
-                                               Geom64& G) {
+// the float32 pipes.  (u, v): origin texel coordinates (float); hp: origin height.
+__device__ __forceinline__ void geom_stereo_frame(const Tile& T, float uf, float vf, DF hp,
+                                                  GeomDF& F) {
     const DF g = { T.g_hi, T.g_lo };
     const DF Xp = df_mul(g, df_two_sum(uf, -T.cx_f));
     const DF Yp = df_mul(g, df_two_sum(vf, -T.cy_f));
@@ -466,35 +472,49 @@ __device__ __forceinline__ void geom_stereo_df(const Tile& T, float uf, float vf
     const DF den = df_add(fr, r2);
     const DF iden = df_div(DF{ 1.0f, 0.0f }, den);
     const DF R4 = { 4.0f * T.R_f, 4.0f * T.R_lo };
-    const DF nx = df_mul(df_mul(R4, Xp), iden), ny = df_mul(df_mul(R4, Yp), iden);
-    const DF nz = df_mul(df_add(fr, df_neg(r2)), iden);
+    F.n[0] = df_mul(df_mul(R4, Xp), iden);
+    F.n[1] = df_mul(df_mul(R4, Yp), iden);
+    F.n[2] = df_mul(df_add(fr, df_neg(r2)), iden);
     const DF sx = { T.sx_f, T.sx_lo }, sy = { T.sy_f, T.sy_lo }, sz = { T.sz_f, T.sz_lo };
-    const DF se = df_add(df_add(df_mul(nx, sx), df_mul(ny, sy)), df_mul(nz, sz));
-    const DF rho = df_add(DF{ T.R_f, T.R_lo }, hp);
-    const DF irho = df_div(DF{ 1.0f, 0.0f }, rho);
+    F.se = df_add(df_add(df_mul(F.n[0], sx), df_mul(F.n[1], sy)), df_mul(F.n[2], sz));
+    F.rho = df_add(DF{ T.R_f, T.R_lo }, hp);
+    F.irho = df_div(DF{ 1.0f, 0.0f }, F.rho);
     // a0 = rho (1 + n_z) = 2 fr rho / (fr + r2)
-    const DF ia0 = df_div(df_mul(irho, den), DF{ 2.0f * fr.hi, 2.0f * fr.lo });
+    F.ia0 = df_div(df_mul(F.irho, den), DF{ 2.0f * fr.hi, 2.0f * fr.lo });
     const DF k2 = { T.k2_hi, T.k2_lo };
     const DF dk = df_mul(DF{ T.delta_hi, T.delta_lo }, k2);
-    const DF kr = df_mul(df_mul(k2, rho), df_mul(ia0, ia0));
+    const DF kr = df_mul(df_mul(k2, F.rho), df_mul(F.ia0, F.ia0));
+    F.Au = df_mul(df_mul(dk, sx), F.ia0);
+    F.Av = df_mul(df_mul(dk, sy), F.ia0);
+    F.Bu = df_mul(kr, F.n[0]);
+    F.Bv = df_mul(kr, F.n[1]);
+    F.b = DF{ 0.0f, 0.0f };
+}
+
+// The same as FP64 values (the two words summed).
+__device__ __forceinline__ void geom_stereo_df(const Tile& T, float uf, float vf, DF hp,
+                                               Geom64& G) {
+    GeomDF F;
+    geom_stereo_frame(T, uf, vf, hp, F);
     G.up = (double)uf;
     G.vp = (double)vf;
     G.hp = df_to_double(hp);
-    G.nhat[0] = df_to_double(nx);
-    G.nhat[1] = df_to_double(ny);
-    G.nhat[2] = df_to_double(nz);
-    G.sin_e = df_to_double(se);
-    G.rho = df_to_double(rho);
-    G.inv_rho = df_to_double(irho);
-    G.inv_a0 = df_to_double(ia0);
-    G.Au = df_to_double(df_mul(df_mul(dk, sx), ia0));
-    G.Av = df_to_double(df_mul(df_mul(dk, sy), ia0));
-    G.Bu = df_to_double(df_mul(kr, nx));
-    G.Bv = df_to_double(df_mul(kr, ny));
+    G.nhat[0] = df_to_double(F.n[0]);
+    G.nhat[1] = df_to_double(F.n[1]);
+    G.nhat[2] = df_to_double(F.n[2]);
+    G.sin_e = df_to_double(F.se);
+    G.rho = df_to_double(F.rho);
+    G.inv_rho = df_to_double(F.irho);
+    G.inv_a0 = df_to_double(F.ia0);
+    G.Au = df_to_double(F.Au);
+    G.Av = df_to_double(F.Av);
+    G.Bu = df_to_double(F.Bu);
+    G.Bv = df_to_double(F.Bv);
     G.b = 0.0;
     // |z of unit(n x s)| (image circle curvature; a float32 bound is enough)
-    const float cxf = ny.hi * sz.hi - nz.hi * sy.hi, cyf = nz.hi * sx.hi - nx.hi * sz.hi;
-    const float czf = nx.hi * sy.hi - ny.hi * sx.hi;
+    const float cxf = F.n[1].hi * T.sz_f - F.n[2].hi * T.sy_f;
+    const float cyf = F.n[2].hi * T.sx_f - F.n[0].hi * T.sz_f;
+    const float czf = F.n[0].hi * T.sy_f - F.n[1].hi * T.sx_f;
     const float cnf = sqrtf(cxf * cxf + cyf * cyf + czf * czf);
     G.nz_cross = cnf > 0.0f ? (double)(fabsf(czf) / cnf) : 0.0;
 }
@@ -518,6 +538,63 @@ __device__ __forceinline__ DF origin_height_df(const Tile& T, float uf, float vf
                                h11));
     href = h00;
     return df_add(acc, DF{ lift, 0.0f });
+}
+
+// geom64's fields (gnomonic) likewise.
+__device__ __forceinline__ void geom_gnomonic_frame(const Tile& T, float uf, float vf, DF hp,
+                                                    GeomDF& F) {
+    const DF g = { T.g_hi, T.g_lo };
+    const DF Xp = df_mul(g, df_two_sum(uf, -T.cx_f));
+    const DF Yp = df_mul(g, df_two_sum(vf, -T.cy_f));
+    const DF m2 = df_add(df_add(df_mul(Xp, Xp), df_mul(Yp, Yp)), DF{ T.RR_hi, T.RR_lo });
+    const DF m = df_sqrt(m2);
+    const DF sx = { T.sx_f, T.sx_lo }, sy = { T.sy_f, T.sy_lo }, sz = { T.sz_f, T.sz_lo };
+    const DF R = { T.R_f, T.R_lo };
+    F.rho = df_add(R, hp);
+    F.se = df_div(df_add(df_add(df_mul(Xp, sx), df_mul(Yp, sy)), df_mul(R, sz)), m);
+    const DF f = df_mul(DF{ T.delta_hi, T.delta_lo }, df_div(m, F.rho));
+    const DF k = df_mul(f, DF{ T.igR_hi, T.igR_lo });
+    F.Au = df_mul(k, df_add(DF{ T.Rsx_hi, T.Rsx_lo }, df_neg(df_mul(sz, Xp))));
+    F.Av = df_mul(k, df_add(DF{ T.Rsy_hi, T.Rsy_lo }, df_neg(df_mul(sz, Yp))));
+    F.b = df_mul(f, DF{ T.szR_f, T.szR_lo });
+}
+
+// floor of a float-float value
+__device__ __forceinline__ int32_t df_floor(DF x) {
+    const float f = floorf(x.hi);
+    return (int32_t)f - ((x.hi == f && x.lo < 0.0f) ? 1 : 0);
+}
+
+// Cost of sample j in float-float (leaf_cost64's terms): heights to ~1e-9 m and
+// positions to ~1e-9 texel at the distances of a tile, an error of ~1e-10 rad at
+// the first sample and less beyond, below float32's own rounding of the light.
+__device__ __forceinline__ float leaf_cost_df(const Tile& T, const GeomDF& F, float uf, float vf,
+                                              DF hp, int32_t j, bool stereo) {
+    const DF jd = { (float)j, 0.0f };
+    const DF t = df_mul_f(DF{ T.delta_hi, T.delta_lo }, (float)j);
+    const DF w = df_mul(t, df_add(df_mul(DF{ 2.0f * F.rho.hi, 2.0f * F.rho.lo }, F.se), t));
+    const DF rise = df_div(w, df_add(F.rho, df_sqrt(df_add(df_mul(F.rho, F.rho), w))));
+    DF du, dv;
+    if (!stereo) {
+        const DF tau = df_div(jd, df_add(DF{ 1.0f, 0.0f }, df_mul(F.b, jd)));
+        du = df_mul(F.Au, tau);
+        dv = df_mul(F.Av, tau);
+    } else {
+        const DF ws = df_add(rise, df_mul(t, DF{ T.sz_f, T.sz_lo }));
+        const DF id = df_div(DF{ 1.0f, 0.0f }, df_add(DF{ 1.0f, 0.0f }, df_mul(ws, F.ia0)));
+        du = df_mul(df_add(df_mul(F.Au, jd), df_neg(df_mul(F.Bu, ws))), id);
+        dv = df_mul(df_add(df_mul(F.Av, jd), df_neg(df_mul(F.Bv, ws))), id);
+    }
+    const DF U = df_add(du, DF{ uf, 0.0f }), V = df_add(dv, DF{ vf, 0.0f });
+    const int32_t i0 = min(max(df_floor(U), 0), T.nx - 2), j0 = min(max(df_floor(V), 0), T.ny - 2);
+    const DF fu = df_add(U, DF{ -(float)i0, 0.0f }), fv = df_add(V, DF{ -(float)j0, 0.0f });
+    const float* p = T.h + (int64_t)j0 * T.pitch + i0;
+    const float h00 = p[0], h10 = p[1], h01 = p[T.pitch], h11 = p[T.pitch + 1];
+    const DF top = df_add(df_mul(fu, df_two_sum(h10, -h00)), DF{ h00, 0.0f });
+    const DF bot = df_add(df_mul(fu, df_two_sum(h11, -h01)), DF{ h01, 0.0f });
+    const DF hb = df_add(df_mul(fv, df_add(bot, df_neg(top))), top);
+    const DF c = df_div(df_add(df_add(hp, df_neg(hb)), rise), t);
+    return c.hi;
 }
 
 // 1/rho^2 from 1/(2 rho) (gnomonic setup; recomputed when a parked ray is loaded)

@@ -233,12 +233,6 @@ __device__ __forceinline__ void view_image_df(const Tile& T, const Cam& cm, cons
     v = df_add(df_mul(y, k), DF{ T.cy_f, 0.0f });
 }
 
-// floor of a float-float value of at most 2^17
-__device__ __forceinline__ int32_t df_floor(DF x) {
-    const float f = floorf(x.hi);
-    return (int32_t)f - ((x.hi == f && x.lo < 0.0f) ? 1 : 0);
-}
-
 __device__ __forceinline__ ViewPtDF view_pt_df(const Tile& T, const Cam& cm, const ViewDir& r, DF tau) {
     ViewPtDF p;
     float den;
