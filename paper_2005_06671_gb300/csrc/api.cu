@@ -288,10 +288,10 @@ ss_status shadow_common(FwdKind kind, const ss_heightfield* hf, const float* mip
     // to 15x (100 k scattered points: 3.3 -> 0.22 ms); the same within 5 us below
     // 1,500 rays.  The walks stay for callers that set a shape.
     if (descent && takes_packets(params, J))
-        a.pk_len = ss::pk_strip_len(rays->mode == SS_RAYS_GRID
-                                        ? ss::pk_grid_strips(hf->nx, hf->ny, 1)
-                                        : (n + 31) / 32,
-                                    light_only);
+        a.pk = ss::pk_shape(rays->mode == SS_RAYS_GRID
+                                ? ss::pk_grid_strips(hf->nx, hf->ny, ss::PkShape{ 32, 1 })
+                                : (n + 31) / 32,
+                            rays->mode != SS_RAYS_GRID, light_only);
     cudaError_t e = kind == FwdKind::Descent
                         ? ss::launch_dp_forward(a, block, (cudaStream_t)stream)
                         : ss::launch_uniform_forward(a, block, (cudaStream_t)stream);
@@ -371,15 +371,15 @@ ss_status batch_prepare(const ss_batch_item* items, int32_t n, const ss_params* 
         d.tile_w = tile_w;
         n_poly += d.poly;
         packets = packets && takes_packets(params, J);
-        n_packets += ss::pk_grid_strips(it.hf.nx, it.hf.ny, 1);
+        n_packets += ss::pk_grid_strips(it.hf.nx, it.hf.ny, ss::PkShape{ 32, 1 });
     }
     // packets of rays (batch_packet.cu) unless a launch shape is asked for; one
     // form of the rise serves a launch, so a batch that mixes both takes chunks
-    const int32_t pk_len = packets && (n_poly == 0 || n_poly == n)
-                               ? ss::pk_strip_len(n_packets, batch_light) : 0;
+    const ss::PkShape pk = packets && (n_poly == 0 || n_poly == n)
+                               ? ss::pk_shape(n_packets, false, batch_light) : ss::PkShape{ 32, 0 };
     for (int32_t i = 0; i < n; ++i)
         prefix[i + 1] = prefix[i] +
-                        (pk_len > 0 ? ss::pk_grid_strips(descs[i].T.nx, descs[i].T.ny, pk_len)
+                        (pk.len > 0 ? ss::pk_grid_strips(descs[i].T.nx, descs[i].T.ny, pk)
                                     : ss::chunk_count(descs[i].n_rays, descs[i].T.nx,
                                                       descs[i].T.ny, chunk, tile_w));
     unsigned long long* counter;
@@ -399,7 +399,7 @@ ss_status batch_prepare(const ss_batch_item* items, int32_t n, const ss_params* 
                                          : (B.args.light_only ? 1 : kDefaultStrip);
     B.args.colseed = (params->strip_len == 0 && !B.args.light_only && tile_w > 0) ? 1 : 0;
     B.args.seed_w = params->seed_width > 0 ? params->seed_width : 1;   // grid rays
-    B.args.pk_len = pk_len;
+    B.args.pk = pk;
     B.args.poly = n_poly == n ? 1 : 0;
     B.args.lane_leaves = (params->flags & SS_FLAG_LANE_LEAVES) ? 1 : 0;
     return SS_OK;

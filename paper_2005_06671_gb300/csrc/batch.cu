@@ -548,7 +548,7 @@ void batch_layout(void* ws, int32_t n_items, unsigned long long** counter, Batch
 }
 
 cudaError_t launch_batch_forward(const BatchArgs& a, int block, bool count, cudaStream_t s) {
-    if (a.pk_len > 0) return launch_batch_packets(a, count, s);
+    if (a.pk.len > 0) return launch_batch_packets(a, count, s);
     const size_t smem = (size_t)(block / 32) *
                             (sizeof(BatchItemDesc) + sizeof(WarpSched) + 3 * kBatchSeedW * sizeof(int32_t)) +
                         (size_t)block * sizeof(LaneRay);

@@ -1,7 +1,7 @@
 // The batch's default kernel: packets of rays (ss_packet.cuh) from one queue over
 // all instances.
 //
-// The queue hands out strips of pk_len packets (consecutive strips of one
+// The queue hands out strips of packets (consecutive strips of one
 // instance are neighbours on its tile).  A warp keeps a copy of its instance's
 // descriptor in shared memory and walks its strip as the single-tile kernel
 // does; all its lanes work on one packet at a time, so nothing of another
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kPkThreads, SS_PK_MIN_BLOCKS) batch_packet_ker
         }
         pk_grid_strip<kCount, kPoly, kLight, false>(D.T, D.L, D.levels, grid_rays, D.O,
                                                     (uint32_t)(q - __ldg(a.chunk_prefix + item)),
-                                                    a.pk_len, span, s_w[threadIdx.x >> 5], lane);
+                                                    a.pk, span, s_w[threadIdx.x >> 5], lane);
     }
 }
 
@@ -80,9 +80,9 @@ __global__ void __launch_bounds__(256) batch_refine_kernel(const BatchArgs a) {
         const uint32_t nbx = (uint32_t)(nx + kPkCols - 1) / kPkCols;
         const uint32_t strip = (uint32_t)(q - __ldg(a.chunk_prefix + item)), band = strip / nbx;
         const int32_t x = (int32_t)(strip - band * nbx) * kPkCols + (threadIdx.x & (kPkCols - 1));
-        const int64_t y0 = (int64_t)band * a.pk_len * kPkRows + (threadIdx.x & 31) / kPkCols;
-        for (int k = 0; k < a.pk_len; ++k) {
-            const int64_t y = y0 + k * kPkRows;
+        const int32_t rows = a.pk.rays / kPkCols * a.pk.len;
+        for (int32_t k = (threadIdx.x & 31) / kPkCols; k < rows; k += kPkRows) {
+            const int64_t y = (int64_t)band * rows + k;
             if (x >= nx || y >= ny) break;
             const int64_t r = y * nx + x;
             if (D.O.light[r] == kLightPending) {

@@ -349,9 +349,20 @@ int device_sm_count() {
 // seed.  Sum over three suns, ms, with 4 / 2 waves: 1024^2 1.47 / 1.43, light-only 1.21 /
 // 0.98; 1531 x 1021 1.97 / 2.03, 1.46 / 1.34; 2048^2 5.16 / 5.53, 3.21 / 3.15.  At most 16:
 // 4096^2 20.5 and 11.6 with 16, 20.8 and 12.4 with 8, 20.7 and 11.5 with 32.
-int32_t pk_strip_len(int64_t packets, bool light) {
-    const int64_t len = packets / ((int64_t)device_sm_count() * 32 * (light ? 2 : 4));
-    return (int32_t)(len < 1 ? 1 : len > kPkMaxLen ? kPkMaxLen : len);
+// Launches of few packets take packets of 16 or 8 rays: more warps, each with a shorter
+// chain of passes, against less sharing.  us with 32 / 16 / 8 rays: tiles of 200^2 56 / 40 /
+// 37, 256^2 60 / 47 / 49, 384^2 93 / 75 / 91, 512^2 134 / 122 / 161; light-only 300^2 57 / 52 / 64,
+// 384^2 70 / 73 / 95; scattered points 1,000 98 / 54 / 37, 60 k 137 / 120 / 118, 400 k 498 / 456 /
+// 492; view points 45 k 426 / 281 / 219, 518 k 732 / 624 / 799, 1.04 M 1861 / 1991 / 2866.
+PkShape pk_shape(int64_t packets, bool list, bool light) {
+    const int64_t warps = (int64_t)device_sm_count() * 32;   // resident
+    const int64_t len = packets / (warps * (light ? 2 : 4));
+    PkShape k;
+    k.len = (int32_t)(len < 1 ? 1 : len > kPkMaxLen ? kPkMaxLen : len);
+    const int64_t few = list ? 4 * warps : light ? warps * 3 / 4 : warps * 7 / 4;
+    const int64_t fewer = list ? warps * 2 / 5 : warps / 4;
+    k.rays = packets <= fewer ? 8 : packets <= few ? 16 : 32;
+    return k;
 }
 
 // Grid-stride kernels: one wave of resident blocks (occupancy x SMs), fewer

@@ -5,7 +5,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
-#include "ss_device.cuh"
+#include "ss_launch.h"
 
 namespace ss {
 
@@ -37,7 +37,7 @@ struct BatchArgs {
     int32_t colseed;                // rectangular chunks: single rays, column seeds
     int32_t seed_w;                 // half-width of a seed window
     int32_t lane_leaves;            // SS_FLAG_LANE_LEAVES: leaves in the walking lane
-    int32_t pk_len;                 // > 0: packets of rays, chunks are strips of so many
+    PkShape pk;                     // len > 0: packets of rays, chunks are strips of them
     int32_t poly;                   // packets: the rise series is valid for every ray
 };
 

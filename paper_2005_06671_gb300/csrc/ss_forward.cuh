@@ -516,7 +516,7 @@ static void launch_packet(const FwdArgs& a, cudaStream_t s);
 template <bool C, bool G, bool P, bool L, bool S>
 struct DpLaunch {
     static cudaError_t go(const FwdArgs& a, int grid, int block, cudaStream_t s) {
-        bool tasks = a.pk_len > 0;
+        bool tasks = a.pk.len > 0;
         if (tasks) launch_packet<C, G, P, L, S>(a, s);
         if constexpr (!L) {
             if (!tasks && use_task_descent(a, G, S, L)) {

@@ -21,6 +21,20 @@ struct MipLayout {
 
 bool mip_layout(int32_t nx, int32_t ny, MipLayout* L);
 
+// Packet descent (ss_packet.cuh): rays of a packet (32, fewer for launches that would
+// not fill the GPU) and packets a warp takes one after the other.  Grid packets are
+// rectangles of kPkCols columns, strips run down the tile.
+struct PkShape {
+    int32_t rays, len;   // len = 0: another kernel
+};
+constexpr int kPkCols = 8, kPkRows = 4;
+inline int64_t pk_grid_strips(int32_t nx, int32_t ny, PkShape k) {
+    const int64_t rows = (int64_t)(k.rays / kPkCols) * k.len;
+    return (int64_t)((nx + kPkCols - 1) / kPkCols) * ((ny + rows - 1) / rows);
+}
+constexpr int kPkMaxLen = 16;
+PkShape pk_shape(int64_t packets, bool list, bool light);   // packets of 32 rays in the launch
+
 struct FwdArgs {
     Tile T;
     Pyramid P;
@@ -36,21 +50,11 @@ struct FwdArgs {
     int32_t strip;            // descent: rays per strip (1 = no seeding)
     int32_t colseed;          // descent, grid rays in rectangles: column seeds
     int32_t seed_w;           // descent: half-width of a seed window
-    int32_t pk_len;           // packet descent: packets per warp (0: another kernel)
+    PkShape pk;               // packet descent
 };
 
 constexpr int32_t kColSeedMaxW = 512;    // widest rectangle with a column-seed table
 constexpr int32_t kListSeedCols = 512;   // listed rays: columns of consecutive ids
-
-// Packet descent (ss_packet.cuh): texels of a grid packet, strips of `len` packets
-// one below the other, and how many packets a warp takes.
-constexpr int kPkCols = 8, kPkRows = 4;
-inline int64_t pk_grid_strips(int32_t nx, int32_t ny, int32_t len) {
-    return (int64_t)((nx + kPkCols - 1) / kPkCols) *
-           ((ny + (int64_t)kPkRows * len - 1) / ((int64_t)kPkRows * len));
-}
-constexpr int kPkMaxLen = 16;
-int32_t pk_strip_len(int64_t packets, bool light);
 
 struct BwdArgs {
     Tile T;

@@ -407,14 +407,13 @@ __device__ __forceinline__ void pk_push_nodes(Warp& W, PkRings& Q, bool mine, in
 }
 
 // The descent of one packet whose rays are in W and whose seeds wait as leaf
-// tasks.  q: the lane's own ray's test; jh: its last usable sample (0: no ray);
-// csat: light-only, the cost that saturates.  On return every sample that could
-// win has been evaluated.  One loop with one copy of each stage: unrolled into
+// tasks.  jh: the last usable sample of the lane's own ray (0: no ray).  On return
+// every sample that could win has been evaluated.  One loop with one copy of each stage: unrolled into
 // its callers the code outgrew the instruction cache (the top stall).
 template <bool kCount, bool kPoly, bool kLight, bool kStereo, class Warp>
 __device__ __forceinline__ void pk_descend(const Tile& T, const LevelTab& L, int32_t levels,
-                                           Warp& W, const PkUnion<kStereo>& U, const PkTest& q,
-                                           int32_t jh, float csat, PkRings& Q, int lane) {
+                                           Warp& W, const PkUnion<kStereo>& U, int32_t jh,
+                                           PkRings& Q, int lane) {
     const float d = T.delta_f;
     const int32_t jmax = __reduce_max_sync(kFull, jh);
     int32_t s = 0, sn = 0;              // next batch of top blocks; the current top block
@@ -463,6 +462,10 @@ __device__ __forceinline__ void pk_descend(const Tile& T, const LevelTab& L, int
             if (kCount) atomicAdd(&W.cnt[0][lane], 1);
         }
         const float dt = (float)(1 << log) * d;
+        // (the lane's own test is read back here: kept in registers across the loop it was
+        // spilled, and one build got it wrong)
+        const float4 qv = W.ray[2][lane];
+        const PkTest q = { qv.y, qv.z, qv.w };
         // curvature term of the block length (0.1%: the roundings of t)
         const float hg = __fmaf_rn(-0.2503f * q.c * dt, dt, q.hg);
         const float best = key_cost(W.key[lane]);
@@ -471,7 +474,7 @@ __device__ __forceinline__ void pk_descend(const Tile& T, const LevelTab& L, int
         W.M[lane] = M;
         __syncwarp();
         // blocks that hold usable samples of the lane's ray
-        if (kLight && best <= -csat) jh = 0;
+        if (kLight && best <= -W.csat[lane]) jh = 0;
         const int32_t nv = nodes && jh > base ? min((jh - base + (1 << log) - 1) >> log, 32) : 0;
         const int32_t ng = min((jmax - base + (1 << log) - 1) >> log, 32);   // of any ray's
         const float tb = (float)base * d;
@@ -532,15 +535,13 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
                                           const Rays& R, const Outputs& O, int64_t ray, bool live,
                                           float span, Warp& W, int lane,
                                           int32_t& prev_j, float& pu, float& pv) {
-    PkTest q;
     PkUnion<kStereo> U;
     int32_t jh, jc = -1;
     float csat = INFINITY, u0, v0, au, av;
     {
         RayF rf;
         setup_ray<kGrid, kLight, kStereo>(T, R, ray, span, rf);
-        q = pk_test<kGrid>(T, rf, span);
-        pk_store(W, lane, rf, q);
+        pk_store(W, lane, rf, pk_test<kGrid>(T, rf, span));
         jh = live && rf.j_lo <= rf.j_hi ? rf.j_hi : 0;
         if (kLight) csat = rf.c_sat;
         if (prev_j > 0)
@@ -549,7 +550,7 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
         v0 = rf.v0;
         au = rf.au;
         av = rf.av;
-        if constexpr (kGrid) {   // (8 x 4 texels, the last lane's the far corner)
+        if constexpr (kGrid) {   // (a rectangle: the last lane's is the far corner)
             U.u0[0] = __shfl_sync(kFull, rf.u0, 0);
             U.v0[0] = __shfl_sync(kFull, rf.v0, 0);
             U.u0[1] = __shfl_sync(kFull, rf.u0, 31);
@@ -598,7 +599,7 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
         near_seed(jh > 0, jc);
         sparse_seeds(!kLight && jh > 0 && jc < 0);
         __syncwarp();
-        pk_descend<kCount, kPoly, kLight, kStereo>(T, L, levels, W, U, q, jh, csat, Q, lane);
+        pk_descend<kCount, kPoly, kLight, kStereo>(T, L, levels, W, U, jh, Q, lane);
     } else {
         // Listed rays that are neighbours (a view's): every fourth ray first, seeded as
         // above and around each other's minima, then the others around the minima of
@@ -636,33 +637,35 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
     __syncwarp();
 }
 
-// A strip of `len` grid packets, 8 x 4 texels each, one below the other; the last
-// row of one seeds the next.  Strips run row by row over the tile.
+// A strip of k.len grid packets of 8 columns, one below the other; the last row of
+// one seeds the next.  Strips run row by row over the tile.  Lanes without a ray
+// repeat one of the packet's.
 template <bool kCount, bool kPoly, bool kLight, bool kStereo, class Warp>
 __device__ __forceinline__ void pk_grid_strip(const Tile& T, const LevelTab& L, int32_t levels,
                                               const Rays& R, const Outputs& O, uint32_t strip,
-                                              int32_t len, float span, Warp& W, int lane) {
+                                              PkShape sh, float span, Warp& W, int lane) {
     const uint32_t nbx = (uint32_t)(T.nx + kPkCols - 1) / kPkCols;
     const uint32_t band = strip / nbx;
     const int32_t x = (int32_t)(strip - band * nbx) * kPkCols + (lane & (kPkCols - 1));
-    const int64_t y0 = (int64_t)band * len * kPkRows;
+    const int32_t rows = sh.rays / kPkCols, row = min(lane / kPkCols, rows - 1);
+    const int64_t y0 = (int64_t)band * sh.len * rows;
     int32_t prev_j = -1;
     float pu = 0.0f, pv = 0.0f;
-    for (int k = 0; k < len && y0 + k * kPkRows < T.ny; ++k) {
-        const int32_t y = (int32_t)y0 + k * kPkRows + lane / kPkCols;
-        const bool live = x < T.nx && y < T.ny;
+    for (int k = 0; k < sh.len && y0 + k * rows < T.ny; ++k) {
+        const int32_t y = (int32_t)y0 + k * rows + row;
+        const bool live = lane < sh.rays && x < T.nx && y < T.ny;
         const int64_t ray = (int64_t)min(y, T.ny - 1) * T.nx + min(x, T.nx - 1);
         pk_packet<kCount, true, kPoly, kLight, kStereo>(T, L, levels, R, O, ray, live, span, W,
                                                         lane, prev_j, pu, pv);
-        const int below = 32 - kPkCols + (lane & (kPkCols - 1));   // the last row's column
+        const int below = sh.rays - kPkCols + (lane & (kPkCols - 1));   // the last row's column
         prev_j = __shfl_sync(kFull, prev_j, below);
         pu = __shfl_sync(kFull, pu, below);
         pv = __shfl_sync(kFull, pv, below);
     }
 }
 
-// Each warp takes a strip of a.pk_len packets (listed rays: 32 consecutive ids
-// each).
+// Each warp takes a strip of a.pk.len packets (listed rays: a.pk.rays consecutive
+// ids each).
 template <bool kCount, bool kGrid, bool kPoly, bool kLight, bool kStereo>
 __global__ void __launch_bounds__(kPkThreads, SS_PK_MIN_BLOCKS)
 dp_packet_kernel(const __grid_constant__ FwdArgs a) {
@@ -680,16 +683,17 @@ dp_packet_kernel(const __grid_constant__ FwdArgs a) {
     auto& W = s_w[threadIdx.x >> 5];
     if constexpr (kGrid) {
         pk_grid_strip<kCount, kPoly, kLight, kStereo>(a.T, s_lev, a.P.levels, a.R, a.O, strip,
-                                                      a.pk_len, span, W, lane);
+                                                      a.pk, span, W, lane);
     } else {
         int32_t prev_j = -1;
         float pu = 0.0f, pv = 0.0f;
-        const int64_t first = (int64_t)strip * a.pk_len * 32;
-        for (int k = 0; k < a.pk_len && first + k * 32 < a.R.n; ++k) {
-            const int64_t id = first + k * 32 + lane;
-            pk_packet<kCount, kGrid, kPoly, kLight, kStereo>(a.T, s_lev, a.P.levels, a.R, a.O,
-                                                             min(id, a.R.n - 1), id < a.R.n, span,
-                                                             W, lane, prev_j, pu, pv);
+        const int32_t m = a.pk.rays, own = min(lane, m - 1);
+        const int64_t first = (int64_t)strip * a.pk.len * m;
+        for (int k = 0; k < a.pk.len && first + k * m < a.R.n; ++k) {
+            const int64_t id = first + k * m + own;
+            pk_packet<kCount, kGrid, kPoly, kLight, kStereo>(
+                a.T, s_lev, a.P.levels, a.R, a.O, min(id, a.R.n - 1), lane < m && id < a.R.n,
+                span, W, lane, prev_j, pu, pv);
         }
     }
 }
@@ -697,8 +701,8 @@ dp_packet_kernel(const __grid_constant__ FwdArgs a) {
 template <bool C, bool G, bool P, bool L, bool S>
 static void launch_packet(const FwdArgs& a, cudaStream_t s) {
     const int64_t n = a.R.mode == 0 ? (int64_t)a.T.nx * a.T.ny : a.R.n;
-    const int64_t strips = a.R.mode == 0 ? pk_grid_strips(a.T.nx, a.T.ny, a.pk_len)
-                                         : (n + 32 * (int64_t)a.pk_len - 1) / (32 * (int64_t)a.pk_len);
+    const int64_t per = (int64_t)a.pk.rays * a.pk.len;
+    const int64_t strips = a.R.mode == 0 ? pk_grid_strips(a.T.nx, a.T.ny, a.pk) : (n + per - 1) / per;
     const int64_t grid = (strips + kPkThreads / 32 - 1) / (kPkThreads / 32);
     dp_packet_kernel<C, G, P, L, S><<<(unsigned)grid, kPkThreads, 0, s>>>(a);
 }

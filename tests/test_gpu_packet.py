@@ -37,10 +37,14 @@ def _same(hf, sun, lmax, **kw):
     b = ss.ss_shadow_uniform(hf, mip, sun, lmax, early_exit=False, **kw)
     for k in ("argmin", "cost", "light"):
         assert torch.equal(a[k], b[k]), k
-    lit = ss.ss_shadow_forward(hf, mip, sun, lmax, light_only=True, **kw)
-    assert torch.equal(lit["light"], b["light"])
+    c = ss.ss_shadow_forward(hf, mip, sun, lmax, count_samples=True, **kw)
+    for k in ("argmin", "cost", "light"):
+        assert torch.equal(c[k], b[k]), k
     pen = (b["light"] > 0) & (b["light"] < 1)
-    assert torch.equal(lit["argmin"][pen], b["argmin"][pen])
+    for count in (False, True):
+        lit = ss.ss_shadow_forward(hf, mip, sun, lmax, light_only=True, count_samples=count, **kw)
+        assert torch.equal(lit["light"], b["light"])
+        assert torch.equal(lit["argmin"][pen], b["argmin"][pen])
     return b
 
 
@@ -51,6 +55,24 @@ def test_grid_shapes(proj, nx, ny, pad):
     for elev, az in ((1.0, 120.0), (-1.5, 301.0), (35.0, 10.0)):
         _same(_tile(nx, ny, 20.0, proj, pad=pad), _ss().Sun(math.radians(elev), math.radians(az)),
               20e3)
+
+
+# packets of 8, 16 and 32 rays, and strips of several (chosen by the number of rays)
+@pytest.mark.parametrize("proj", ["gnomonic", "polar_stereo"])
+@pytest.mark.parametrize("nx,ny", [(301, 263), (601, 527), (2053, 2501)])
+def test_grid_packet_sizes(proj, nx, ny):
+    for elev, az in ((1.0, 120.0), (38.0, 10.0)):
+        _same(_tile(nx, ny, 20.0, proj), _ss().Sun(math.radians(elev), math.radians(az)), 6e3)
+
+
+@pytest.mark.parametrize("proj", ["gnomonic", "polar_stereo"])
+@pytest.mark.parametrize("n", [100003, 700001])
+def test_many_listed_rays(proj, n):
+    hf = _tile(700, 600, 20.0, proj)
+    rng = np.random.default_rng(n)
+    near = np.stack([np.arange(n) % 5990 * 0.1, np.arange(n) // 5990 * 4.0], 1)
+    for uv in (near, rng.uniform(0.0, 590.0, (n, 2))):
+        _same(hf, _ss().Sun(math.radians(1.3), 0.7), 6e3, uv=torch.from_numpy(uv.astype(np.float32)).cuda())
 
 
 # closed form of the rise (|x| > 1/32), a small sphere, long and short steps, rays of no and of
