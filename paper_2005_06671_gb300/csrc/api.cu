@@ -453,6 +453,8 @@ ss_status backward_common(const ss_heightfield* hf, const ss_rays* rays, const s
     a.grad_pitch = hf->pitch;
     a.grad_sun = grad_sun;
     a.status = status;
+    a.inv_alpha = 1.0 / a.T.alpha;
+    a.img_scale = (hf->projection == SS_PROJ_GNOMONIC ? 1.0 : 2.0) * a.T.R / a.T.g;
     double e = sun->elevation_rad, az = sun->azimuth_rad;
     a.ds_de[0] = -sin(e) * sin(az);
     a.ds_de[1] = -sin(e) * cos(az);

@@ -66,6 +66,7 @@ struct BwdArgs {
     int64_t grad_pitch;
     double* grad_sun;
     double ds_de[3], ds_da[3];
+    double inv_alpha, img_scale;   // 1/alpha; R/g (gnomonic) or 2R/g (stereographic)
     uint32_t* status;           // device status word (non-finite dL/dlight), or null
 };
 
