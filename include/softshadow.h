@@ -250,7 +250,8 @@ ss_status ss_build_maxmip(const ss_heightfield* hf, float* mip, ss_stream_t stre
  * over their texel footprint; blocks whose bound cannot beat the running
  * minimum are skipped; the rest are split until single samples are evaluated.
  * Sample values are float32 in a per-ray local frame (FP64 per-ray setup); the
- * argmin sample of rays with unsaturated light is re-evaluated in FP64.
+ * argmin sample of rays with unsaturated light is re-evaluated to FP64's float32
+ * (float-float arithmetic, FP64 where that leaves the rounding in doubt).
  * mip: device, built by ss_build_maxmip for the same heights. */
 ss_status ss_shadow_forward(const ss_heightfield* hf, const float* mip, const ss_rays* rays,
                             const ss_sun* sun, const ss_params* params,

@@ -6,7 +6,7 @@
 // descriptor in shared memory and walks its strip as the single-tile kernel
 // does; all its lanes work on one packet at a time, so nothing of another
 // instance is ever in flight in the warp.  Penumbra rays are left pending and
-// re-evaluated in FP64 by a second kernel over the same strips, with full warps.
+// re-evaluated by a second kernel over the same strips, with full warps.
 //
 // Bound by instruction issue, as ss_packet.cuh.  16 tiles of 512^2 to 4096^2 (67 M
 // rays, a sun each) take 33.6 ms against 89.9 ms with batch_task_kernel; 16 tiles of
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kPkThreads, SS_PK_MIN_BLOCKS) batch_packet_ker
     }
 }
 
-// FP64 re-evaluation of the rays left pending (refine_kernel over the strips): a
+// Re-evaluation of the rays left pending (refine_kernel over the strips): a
 // block gathers the pending rays of kBatchRefineStrips strips, then every thread
 // takes one.
 constexpr int kBatchRefineStrips = 4;

@@ -288,10 +288,6 @@ __device__ __forceinline__ void pos64(const Tile& T, const Geom64& G, double jd,
     }
 }
 
-__device__ __forceinline__ double cos_elev(const Geom64& G) {
-    return sqrt(fmax(0.0, 1.0 - G.sin_e * G.sin_e));
-}
-
 // Sample index at which u_p + a j/(1 + b j) reaches boundary B (j = (B - u_p) /
 // (a - b (B - u_p))); +inf when it never does.
 __device__ __forceinline__ double cross_j(double p0, double a, double b, double B) {
@@ -565,11 +561,11 @@ __device__ __forceinline__ int32_t df_floor(DF x) {
     return (int32_t)f - ((x.hi == f && x.lo < 0.0f) ? 1 : 0);
 }
 
-// Cost of sample j in float-float (leaf_cost64's terms): heights to ~1e-9 m and
-// positions to ~1e-9 texel at the distances of a tile, an error of ~1e-10 rad at
-// the first sample and less beyond, below float32's own rounding of the light.
-__device__ __forceinline__ float leaf_cost_df(const Tile& T, const GeomDF& F, float uf, float vf,
-                                              DF hp, int32_t j, bool stereo) {
+// Cost of sample j in float-float, (h_p + rise - bilinear height) / t, with heights
+// taken relative to h_p.  err: a bound of its error, 2^-42 of the terms (each comes
+// from at most eight operations that lose up to 2^-45).
+__device__ __forceinline__ DF leaf_cost_df(const Tile& T, const GeomDF& F, float uf, float vf,
+                                           DF hp, int32_t j, bool stereo, float& err) {
     const DF jd = { (float)j, 0.0f };
     const DF t = df_mul_f(DF{ T.delta_hi, T.delta_lo }, (float)j);
     const DF w = df_mul(t, df_add(df_mul(DF{ 2.0f * F.rho.hi, 2.0f * F.rho.lo }, F.se), t));
@@ -590,11 +586,26 @@ __device__ __forceinline__ float leaf_cost_df(const Tile& T, const GeomDF& F, fl
     const DF fu = df_add(U, DF{ -(float)i0, 0.0f }), fv = df_add(V, DF{ -(float)j0, 0.0f });
     const float* p = T.h + (int64_t)j0 * T.pitch + i0;
     const float h00 = p[0], h10 = p[1], h01 = p[T.pitch], h11 = p[T.pitch + 1];
-    const DF top = df_add(df_mul(fu, df_two_sum(h10, -h00)), DF{ h00, 0.0f });
-    const DF bot = df_add(df_mul(fu, df_two_sum(h11, -h01)), DF{ h01, 0.0f });
-    const DF hb = df_add(df_mul(fv, df_add(bot, df_neg(top))), top);
-    const DF c = df_div(df_add(df_add(hp, df_neg(hb)), rise), t);
-    return c.hi;
+    const DF d10 = df_two_sum(h10, -h00), d01 = df_two_sum(h01, -h00);
+    const DF dx = df_add(df_two_sum(h11, -h01), df_neg(d10));
+    const DF rel = df_add(df_two_sum(h00, -hp.hi), DF{ -hp.lo, 0.0f });   // h00 - h_p
+    const DF hb = df_add(df_add(rel, df_mul(fu, d10)), df_mul(fv, df_add(d01, df_mul(fu, dx))));
+    err = 2.3e-13f * (fabsf(rise.hi) + fabsf(rel.hi) + fabsf(d10.hi) + fabsf(d01.hi) +
+                      (fabsf(du.hi) + fabsf(dv.hi)) * (fabsf(d10.hi) + fabsf(d01.hi) + fabsf(dx.hi))) /
+          t.hi;
+    return df_div(df_add(rise, df_neg(hb)), t);
+}
+
+// The same in FP64.
+__device__ __forceinline__ double leaf_cost64(const Tile& T, const Geom64& G, int32_t j, bool stereo) {
+    const double jd = (double)j;
+    const double t = jd * T.delta;
+    double u, v;
+    pos64(T, G, jd, t, u, v, stereo);
+    int32_t i0, j0;
+    double w[4];
+    const double hb = fetch_bilinear64(T.h, T.pitch, T.nx, T.ny, u, v, &i0, &j0, w);
+    return ((G.hp - hb) + rise64(G, t)) / t;
 }
 
 // 1/rho^2 from 1/(2 rho) (gnomonic setup; recomputed when a parked ray is loaded)
@@ -1292,22 +1303,6 @@ __device__ __forceinline__ float probe(const Tile& T, const LevelTab& L, int32_t
     const float num = leaf ? num0 : __fsub_rn(num0, guard);
     const float den_j = (leaf || !(num >= 0.0f)) ? fa : fb;
     return __fmul_rn(num, inv_t(T, den_j));
-}
-
-// ------------------------------------------------------ FP64 re-evaluation
-__device__ __forceinline__ double leaf_cost64(const Tile& T, const Geom64& G, int32_t j,
-                                              bool stereo, double* U = nullptr,
-                                              double* V = nullptr) {
-    const double jd = (double)j;
-    const double t = jd * T.delta;
-    double u, v;
-    pos64(T, G, jd, t, u, v, stereo);
-    if (U) *U = u;
-    if (V) *V = v;
-    int32_t i0, j0;
-    double w[4];
-    const double hb = fetch_bilinear64(T.h, T.pitch, T.nx, T.ny, u, v, &i0, &j0, w);
-    return ((G.hp - hb) + rise64(G, t)) / t;
 }
 
 // ------------------------------------------------ FP64 mapping helpers

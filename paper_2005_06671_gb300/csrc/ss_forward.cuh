@@ -1,5 +1,5 @@
 // Forward kernels (exact max-mip descent, light-only descent, uniform
-// stepping, and the FP64 re-evaluation of penumbra rays), templated on the
+// stepping, and the re-evaluation of penumbra rays), templated on the
 // tile mapping; fwd_gnomonic.cu and fwd_stereo.cu each instantiate one mapping
 // so the two compile in parallel.
 //
@@ -446,21 +446,21 @@ static int pool_grid(const FwdArgs& a) {
 }
 
 // ---------------------------------------------------------------- refine
-// FP64 re-evaluation of the rays the descent left pending (penumbra rays, a
-// few percent).  A block gathers the pending rays of its kRefineRounds x 256
-// ids into shared memory, then every thread takes one: full warps of FP64 work
-// instead of a lane or two inside the walk's services.
+// Re-evaluation (refine_ray) of the rays the descent left pending (penumbra rays, a
+// few percent).  A block gathers the pending rays of its rounds x 256 ids into shared
+// memory, then every thread takes one: full warps instead of a lane or two inside the
+// walk's services.
 constexpr int kRefineRounds = 8;
 
 template <bool kStereo>
-__global__ void __launch_bounds__(256) refine_kernel(const FwdArgs a) {
+__global__ void __launch_bounds__(256) refine_kernel(const FwdArgs a, int rounds) {
     __shared__ int64_t s_ray[256 * kRefineRounds];
     __shared__ int32_t s_cnt;
     const int64_t n = ray_count(a.T, a.R);
-    const int64_t base = (int64_t)blockIdx.x * 256 * kRefineRounds;
+    const int64_t base = (int64_t)blockIdx.x * 256 * rounds;
     if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
-    for (int k = 0; k < kRefineRounds; ++k) {
+    for (int k = 0; k < rounds; ++k) {
         const int64_t r = base + (int64_t)k * 256 + threadIdx.x;
         if (r < n && a.O.light[r] == kLightPending) s_ray[atomicAdd(&s_cnt, 1)] = r;
     }
@@ -531,8 +531,10 @@ struct DpLaunch {
         else
             dp_forward_kernel<C, G, P, S><<<grid, block, 0, s>>>(a);
         const int64_t n = a.R.mode == 0 ? (int64_t)a.T.nx * a.T.ny : a.R.n;
-        const int64_t rb = ((n + 256 * kRefineRounds - 1) / (256 * kRefineRounds));
-        refine_kernel<S><<<(unsigned)rb, 256, 0, s>>>(a);
+        // fewer ids per block where that fills the GPU (256^2: 12 -> 9 us)
+        const int64_t fill = n / ((int64_t)device_sm_count() * 4 * 256);
+        const int rounds = (int)(fill < 1 ? 1 : fill > kRefineRounds ? kRefineRounds : fill);
+        refine_kernel<S><<<(unsigned)((n + 256 * rounds - 1) / (256 * rounds)), 256, 0, s>>>(a, rounds);
         return cudaGetLastError();
     }
 };

@@ -45,12 +45,23 @@ __device__ __forceinline__ float cos_elev_f32(const Tile& T, const Rays& R, int6
     return sqrtf(fmaxf(0.0f, 1.0f - se * se));
 }
 
+// Cost of ray r's sample j in FP64.
+static __device__ __noinline__ float refine_cost64(const Tile& T, const Rays& R, int64_t r, int32_t j,
+                                                   bool stereo) {
+    double up, vp, hp, href, ow[4];
+    int32_t oi0, oj0;
+    ray_origin(T, R, r, up, vp, hp, href, oi0, oj0, ow);
+    Geom64 G;
+    geom64_any(T, up, vp, hp, G, stereo);
+    return (float)leaf_cost64(T, G, j, stereo);
+}
+
 // Re-evaluation of ray r's argmin sample (rays whose light is not saturated): the
-// cost in float-float, the disc formula (Eq. discfrac) in float32 (error < 1e-7 in
-// light).  In FP64, ~180 operations at 1/64 of the float32 rate, refine_kernel took
-// 133 us at 4096^2 (now 55), 38 and 97 us for the Sun and the Earth at 2048^2 (18, 25).
-// Against 64 bits the lights are as far off as before to four digits (mean 2.65e-8 in
-// the penumbra) over 19 tiles and point sets of both mappings.
+// cost to FP64's float32, the disc formula (Eq. discfrac) in float32 (error < 1e-7 in
+// light).  The cost is taken in float-float; where its error could move the
+// rounding to float32 (two rays in a thousand), in FP64.  All in FP64, ~180
+// operations at 1/64 of the float32 rate, refine_kernel took 133 us at 4096^2 (now
+// 81), 38 and 97 us for the Sun and the Earth at 2048^2 (26, 33).
 __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t r,
                                            int32_t bestj, bool stereo, float& light, float& cost) {
     float uf, vf;
@@ -72,7 +83,15 @@ __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t
         geom_stereo_frame(T, uf, vf, hp, F);
     else
         geom_gnomonic_frame(T, uf, vf, hp, F);
-    cost = leaf_cost_df(T, F, uf, vf, hp, bestj, stereo);
+    float err;
+    const DF c = leaf_cost_df(T, F, uf, vf, hp, bestj, stereo, err);
+    // c.hi is the nearest float32 unless c lies within err of the middle between two:
+    // half a step of c.hi away from it (a quarter on the inner side of a power of two)
+    const uint32_t bits = __float_as_uint(c.hi);
+    const float half = __uint_as_float(bits & 0x7f800000u) * 5.9604645e-8f, away = fabsf(c.lo);
+    cost = c.hi;
+    if (!(away < half - err) || ((bits & 0x007fffffu) == 0u && !(away < 0.5f * half - err)))
+        cost = refine_cost64(T, R, r, bestj, stereo);
     const float d = cost * sqrtf(fmaxf(0.0f, 1.0f - F.se.hi * F.se.hi)) / T.alpha_f;
     light = disc_light32(d);
 }
