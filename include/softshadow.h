@@ -215,7 +215,8 @@ typedef struct {
     int32_t* argmin;       /* required: j* (1-based) or -1                     */
     float* cost;           /* optional: c* in rad (+inf when j* = -1), or NULL */
     int32_t* counters;     /* optional [n][2]: (bound probes, leaf samples)
-                              when SS_FLAG_COUNT_SAMPLES is set, or NULL       */
+                              when SS_FLAG_COUNT_SAMPLES is set, or NULL (a
+                              bound shared by a packet counts for one ray)     */
     uint32_t* status;      /* optional device word OR-ed with SS_DEV_* bits
                               (non-finite heights or ray inputs), or NULL      */
 } ss_outputs;
