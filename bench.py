@@ -38,12 +38,12 @@ CONFIG = "mid"
 # One launch of the descent kernel on the 4096x4096 workload, from one ncu capture
 # (profiles/dp_task_grid4096.md; None until taken for the current kernel):
 # dram__bytes_read.sum + dram__bytes_write.sum, and the issue counters
-MID_DP_TRAFFIC_BYTES = 91520000 + 94630400
-MID_DP_ISSUE = {"smsp__inst_executed.sum": 13104574673,
-                "smsp__thread_inst_executed.sum": 312046763948,
-                "sm__cycles_elapsed.avg": 29798239.3, "gpu__time_duration.sum_ns": 14402240}
+MID_DP_TRAFFIC_BYTES = 91290112 + 101828864
+MID_DP_ISSUE = {"smsp__inst_executed.sum": 6007537388,
+                "smsp__thread_inst_executed.sum": 181693707185,
+                "sm__cycles_elapsed.avg": 13416470.58, "gpu__time_duration.sum_ns": 6488928}
 SMS, SMSP_PER_SM = 152, 4
-DESCENT_KERNEL = "dp_task_kernel"
+DESCENT_KERNEL = "dp_packet_kernel"
 
 
 def parse_args(argv=None):
@@ -293,7 +293,7 @@ def run_ours(args):
                    "rays_per_step": n_rays, "l2": "flushed before every timed step (512 MiB write)",
                    "parallelism": f"replicas x{world} (weak)"},
         "clocks": clocks,
-        # per step: the mipmap passes, the descent and its FP64 refine pass
+        # per step: the mipmap passes, the descent and its refine pass
         "gpu_launches": (mip_passes + 2) * args.steps,
         "mip_build_ms": statistics.median(mip_ms),
         "forward_ms": statistics.median(fwd_ms),
