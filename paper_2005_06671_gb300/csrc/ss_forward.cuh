@@ -371,6 +371,10 @@ dp_light_kernel(const __grid_constant__ FwdArgs a) {
 // g(t) = (H(t) - max h - G)/t is non-decreasing and bounds every later
 // sample's cost from below; once g(t_j) >= best no later sample can win.
 // G = 3 guards covers the float32 rounding of both sides.
+// Penumbra rays are left to refine_kernel: float-float inside the services, with a lane
+// or two active and more registers, took 27.3 ms exact / 9.5 ms light-only at 2048^2 and
+// 32.7 / 12.3 ms on a stereographic tile (FP64 there: 26.4 / 9.0, 29.8 / 11.4; now 25.6 /
+// 8.8, 29.4 / 11.2).
 template <bool kCount, bool kGrid, bool kPoly, bool kLight, bool kStereo>
 __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel(const FwdArgs a) {
     __shared__ int32_t s_next;
@@ -390,7 +394,7 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel
         unsigned act = __ballot_sync(kFull, r >= 0 && !done);
         if (act == 0 || (open && __popc(~act) >= a.refill_min)) {
             if (done) {
-                finish_ray<kStereo>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj, 0, nl);
+                finish_ray<kStereo, true>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj, 0, nl);
                 r = -1;
                 done = false;
             }
@@ -410,7 +414,8 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel
                                            0.5f * rf.B * rf.B * rf.inv_2rho);
                     G = 3.0f * kGuardRel * (rf.guard0 + fabsf(hmax_rel) + rb);
                     if (rf.j_hi < rf.j_lo) {   // no usable sample: written at once
-                        finish_ray<kStereo>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj, 0, 0);
+                        finish_ray<kStereo, true>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj,
+                                                  0, 0);
                         r = -1;
                     }
                 }
@@ -446,7 +451,7 @@ static int pool_grid(const FwdArgs& a) {
 }
 
 // ---------------------------------------------------------------- refine
-// Re-evaluation (refine_ray) of the rays the descent left pending (penumbra rays, a
+// Re-evaluation (refine_ray) of the rays the kernels left pending (penumbra rays, a
 // few percent).  A block gathers the pending rays of its rounds x 256 ids into shared
 // memory, then every thread takes one: full warps instead of a lane or two inside the
 // walk's services.
@@ -473,6 +478,15 @@ __global__ void __launch_bounds__(256) refine_kernel(const FwdArgs a, int rounds
         a.O.light[r] = light;
         if (a.O.cost) a.O.cost[r] = cost;
     }
+}
+
+template <bool kStereo>
+static void launch_refine(const FwdArgs& a, cudaStream_t s) {
+    const int64_t n = a.R.mode == 0 ? (int64_t)a.T.nx * a.T.ny : a.R.n;
+    // fewer ids per block where that fills the GPU (256^2: 12 -> 9 us)
+    const int64_t fill = n / ((int64_t)device_sm_count() * 4 * 256);
+    const int rounds = (int)(fill < 1 ? 1 : fill > kRefineRounds ? kRefineRounds : fill);
+    refine_kernel<kStereo><<<(unsigned)((n + 256 * rounds - 1) / (256 * rounds)), 256, 0, s>>>(a, rounds);
 }
 
 #define SS_FWD_CASE(C, G, P, L) \
@@ -530,11 +544,7 @@ struct DpLaunch {
             dp_light_kernel<C, G, P, S><<<grid, block, 0, s>>>(a);
         else
             dp_forward_kernel<C, G, P, S><<<grid, block, 0, s>>>(a);
-        const int64_t n = a.R.mode == 0 ? (int64_t)a.T.nx * a.T.ny : a.R.n;
-        // fewer ids per block where that fills the GPU (256^2: 12 -> 9 us)
-        const int64_t fill = n / ((int64_t)device_sm_count() * 4 * 256);
-        const int rounds = (int)(fill < 1 ? 1 : fill > kRefineRounds ? kRefineRounds : fill);
-        refine_kernel<S><<<(unsigned)((n + 256 * rounds - 1) / (256 * rounds)), 256, 0, s>>>(a, rounds);
+        launch_refine<S>(a, s);
         return cudaGetLastError();
     }
 };
@@ -543,6 +553,7 @@ template <bool C, bool G, bool P, bool L, bool S>
 struct UniLaunch {
     static cudaError_t go(const FwdArgs& a, int grid, int block, cudaStream_t s) {
         uniform_forward_kernel<C, G, P, L, S><<<grid, block, 0, s>>>(a);
+        launch_refine<S>(a, s);
         return cudaGetLastError();
     }
 };
