@@ -332,9 +332,13 @@ __device__ __forceinline__ void pk_node_pass(const Tile& T, const LevelTab& L, i
     bool pa = false, pb = false;
     int32_t s = 0, k = kPkNodeLog;
     int slot = 0;
+    // (the children take the places of the tasks read here, and a vote alone orders no
+    // memory: the barrier does)
+    uint32_t task = 0;
+    if (lane < n)
+        task = kGrid ? W.node[(Q.nh + lane) & (kPkNodeRing - 1)] : W.node[Q.nc - n + lane];
+    if (!kGrid) __syncwarp();
     if (lane < n) {
-        const uint32_t task = kGrid ? W.node[(Q.nh + lane) & (kPkNodeRing - 1)]
-                                    : W.node[Q.nc - n + lane];
         slot = (int)(task & 31u);
         if (!kGrid) k = (int32_t)(task >> 18);
         s = (int32_t)((kGrid ? task : task & 0x3ffffu) >> 5) << kPkNodeLog;
