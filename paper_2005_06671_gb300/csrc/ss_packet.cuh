@@ -349,8 +349,10 @@ __device__ __forceinline__ void pk_node_pass(const Tile& T, const LevelTab& L, i
         const float best = key_cost(W.key[slot]);
         if (kLight && best <= -W.csat[slot]) jh = 0;   // in full umbra: nothing more to find
         const int32_t half = kGrid ? kPkNode / 2 : 1 << (k - 1);
-        const float fs = (float)s, fh = (float)half;
-        const float j0 = fs + 1.0f, j1 = fs + (fh + 0.5f), j2 = fs + 2.0f * fh;
+        // (ends clipped to the last usable sample: past it the image may leave the plane,
+        // 1 + b j <= 0, and a box to there would miss the samples)
+        const float fs = (float)s, fh = (float)half, fj = (float)jh;
+        const float j0 = fs + 1.0f, j1 = fminf(fs + (fh + 0.5f), fj), j2 = fminf(fs + 2.0f * fh, fj);
         const float t0 = j0 * T.delta_f, t1 = j1 * T.delta_f, t2 = j2 * T.delta_f;
         float x0, y0, x1, y1, x2, y2;
         block_end<kStereo>(T, r, j0, t0, kStereo ? rise_of<kPoly>(r, t0) : 0.0f, x0, y0);

@@ -1,0 +1,31 @@
+"""Edges of the packet descent that test_gpu_packet.py's cases do not reach.  Bars as
+there: the bits of uniform stepping."""
+import math
+
+import pytest
+import torch
+
+import paper_2005_06671_gb300 as ss
+
+pytestmark = pytest.mark.gpu
+
+
+# A small sphere, rays diving under a wide tile, a wall far out: past the last usable
+# sample the gnomonic denominator 1 + b j is zero or negative, so a block's far end must
+# not be taken there (the last block then misses the wall, which holds the minimum).
+@pytest.mark.parametrize("n,R,elev,wall,width,height,u0", [
+    (402, 636.0, -41.33, 274, 22, 1043.0, 187), (402, 2894.0, -33.61, 357, 28, 9562.0, 78),
+    (402, 1505.0, -39.85, 298, 24, 1331.0, 153), (402, 2350.0, -37.99, 349, 12, 6881.0, 66),
+    (402, 1811.0, -49.07, 257, 18, 9658.0, 179)])
+def test_block_past_the_last_sample(n, R, elev, wall, width, height, u0):
+    h = torch.zeros((n, n), device="cuda")
+    h[:, wall:wall + width] = height
+    hf = ss.Heightfield(h, 20.0, R)
+    mip = ss.ss_build_maxmip(hf)
+    sun = ss.Sun(math.radians(elev), math.radians(90.0))
+    v = torch.arange(n // 2 - 20, n // 2 + 20, device="cuda")
+    uv = torch.stack([torch.full_like(v, u0), v], 1).float()
+    a = ss.ss_shadow_forward(hf, mip, sun, 20.0 * R, uv=uv)
+    b = ss.ss_shadow_uniform(hf, mip, sun, 20.0 * R, uv=uv, early_exit=False)
+    for k in ("argmin", "cost", "light"):
+        assert torch.equal(a[k], b[k]), k
