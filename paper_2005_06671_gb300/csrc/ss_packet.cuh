@@ -632,6 +632,11 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
             pk_descend_list<kCount, kPoly, kLight, kStereo>(T, L, levels, W, go ? jh : 0, Q, lane);
         }
     }
+    if (kCount) {   // shared bounds counted in lanes without a ray: to the packet's first ray
+        const unsigned mine = __ballot_sync(kFull, live);
+        const unsigned lost = __reduce_add_sync(kFull, live ? 0u : (unsigned)W.cnt[0][lane]);
+        if (mine && lane == __ffs(mine) - 1) W.cnt[0][lane] += (int32_t)lost;
+    }
     const unsigned long long key = W.key[lane];
     const int32_t bj = kLight && key_j(key) == 0 ? -1 : key_j(key);
     if (live)

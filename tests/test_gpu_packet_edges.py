@@ -29,3 +29,28 @@ def test_block_past_the_last_sample(n, R, elev, wall, width, height, u0):
     b = ss.ss_shadow_uniform(hf, mip, sun, 20.0 * R, uv=uv, early_exit=False)
     for k in ("argmin", "cost", "light"):
         assert torch.equal(a[k], b[k]), k
+
+
+# Every bound shared by a packet counts for one of its rays, also where the packet has
+# fewer than 32 (small launches: 8 or 16; the tile's edges).  On flat ground under a high
+# sun the light-only count is known: the packet's blocks of 256 samples, the blocks of 8
+# of the first one, and the two halves of each ray's own first block, none else survives.
+@pytest.mark.parametrize("nx,ny,rows", [(64, 64, 1), (301, 263, 2), (603, 530, 4)])
+def test_counters_hold_every_shared_bound(nx, ny, rows):
+    hf = ss.Heightfield(torch.zeros((ny, nx), device="cuda"), 20.0, 1737.4e3)
+    mip = ss.ss_build_maxmip(hf)
+    kw = dict(step_texels=0.1, count_samples=True)
+    for az in (120.0, 301.0):
+        sun = ss.Sun(math.radians(30.0), math.radians(az))
+        a = ss.ss_shadow_forward(hf, mip, sun, 20e3, light_only=True, **kw)
+        b = ss.ss_shadow_uniform(hf, mip, sun, 20e3, early_exit=False, **kw)
+        jh = b["counters"][:, 1].long()                     # usable samples of the ray
+        py, px = (ny + rows - 1) // rows, (nx + 7) // 8
+        r = torch.arange(nx * ny, device="cuda")
+        packet = (r // nx // rows) * px + r % nx // 8
+        zero = torch.zeros(py * px, dtype=torch.long, device="cuda")
+        jmax = zero.scatter_reduce(0, packet, jh, "amax")
+        want = (jmax + 255) // 256 + ((jmax + 7) // 8).clamp(max=32)
+        want = want.scatter_add(0, packet, 2 * (jh > 0).long())
+        got = zero.scatter_add(0, packet, a["counters"][:, 0].long())
+        assert torch.equal(got, want)
