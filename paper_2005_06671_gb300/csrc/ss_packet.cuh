@@ -315,7 +315,7 @@ __device__ __forceinline__ void pk_leaf_pass(const Tile& T, Warp& W, PkRings& Q,
             const int32_t bj = c[0] == best ? j[0] : c[1] == best ? j[1] : c[2] == best ? j[2] : j[3];
             atomicMin(&W.key[slot], pack_key(best, bj));
         }
-        if (kCount) atomicAdd(&W.cnt[1][slot], 4);
+        if (kCount) atomicAdd(&W.cnt[1][slot], 1 + (j[1] != j[0]) + (j[2] != j[1]) + (j[3] != j[2]));
     }
     Q.lh = (Q.lh + n) & (kPkLeafRing - 1);
     Q.lc -= n;

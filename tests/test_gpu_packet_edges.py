@@ -31,6 +31,14 @@ def test_block_past_the_last_sample(n, R, elev, wall, width, height, u0):
         assert torch.equal(a[k], b[k]), k
 
 
+def _scene(nx, ny, seed=5):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.arange(nx, device="cuda")[None, :]
+    y = torch.arange(ny, device="cuda")[:, None]
+    h = 300.0 * (torch.sin(x / 7.3 + 1.0) * torch.cos(y / 5.1))
+    return (h + 15.0 * torch.randn((ny, nx), device="cuda", generator=gen)).float()
+
+
 # Every bound shared by a packet counts for one of its rays, also where the packet has
 # fewer than 32 (small launches: 8 or 16; the tile's edges).  On flat ground under a high
 # sun the light-only count is known: the packet's blocks of 256 samples, the blocks of 8
@@ -54,3 +62,20 @@ def test_counters_hold_every_shared_bound(nx, ny, rows):
         want = want.scatter_add(0, packet, 2 * (jh > 0).long())
         got = zero.scatter_add(0, packet, a["counters"][:, 0].long())
         assert torch.equal(got, want)
+
+
+# A leaf task clipped to the ray's last sample counts the samples it has: tasks of rays of
+# one or two samples hold one or two (a seed and a leaf task per ray; listed neighbours
+# take up to three seeds more from each other).
+@pytest.mark.parametrize("samples", [1, 2])
+def test_counters_of_clipped_leaf_tasks(samples):
+    hf = ss.Heightfield(_scene(130, 61), 20.0, 1737.4e3)
+    mip = ss.ss_build_maxmip(hf)
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    uv = torch.rand((501, 2), device="cuda", generator=gen) * 59.0
+    for tasks, kw in ((2, dict()), (5, dict(uv=uv))):
+        r = ss.ss_shadow_forward(hf, mip, ss.Sun(math.radians(1.0), 0.3), 10.0 * samples + 1.0,
+                                 count_samples=True, **kw)
+        c = r["counters"][:, 1]
+        assert c.max() <= tasks * samples
+        assert (c[r["argmin"] > 0] >= 1).all()
