@@ -4,9 +4,10 @@
 // calls (series form of the rise) with about half the instructions: the packed
 // operations, floors by round-down additions (exact for |x| < 2^22) whose integer
 // parts are read off the sum's bits, and one test for the clamps at the tile's
-// border, which almost no sample needs.  (A packed multiplication that only feeds a
-// packed addition may be fused with it, .rn or not: the two places where a product
-// is added to something form the product or the sum with scalar instructions.)
+// border, which almost no sample needs.  (A packed multiplication that feeds a packed
+// addition may be fused with it, .rn or not: wherever a rounded product is added to
+// something, the sum, or the product, is formed with scalar instructions, which are not.
+// j * a_hi is exact, fused or not, and the addend of an fma cannot be.)
 #pragma once
 
 #include "ss_device.cuh"
@@ -87,7 +88,9 @@ __device__ __forceinline__ void leaf_cost2(const Tile& T, const RayF& r, int32_t
     const F2 jf = f2(fa, fb), one = f2(1.0f);
     const F2 t = f2_mul(jf, f2(T.delta_f));
     // rise (rise_of<true>)
-    const F2 w = f2_mul(t, f2_add(f2(r.B), t));
+    float t0, t1;
+    f2_get(t, t0, t1);
+    const F2 w = f2_mul(t, f2(__fadd_rn(r.B, t0), __fadd_rn(r.B, t1)));
     const F2 x = f2_mul(w, f2(r.inv_rho2));
     F2 q = f2_fma(x, f2(0.0546875f), f2(-0.078125f));
     q = f2_fma(x, q, f2(0.125f));
@@ -104,9 +107,10 @@ __device__ __forceinline__ void leaf_cost2(const Tile& T, const RayF& r, int32_t
         cu = cv = f2(__fdividef(n0, __fadd_rn(1.0f, d0)), __fdividef(n1, __fadd_rn(1.0f, d1)));
     } else {
         float n0, n1, d0, d1;
-        f2_get(t, d0, d1);
-        const F2 ws = f2_add(rise, f2(__fmul_rn(d0, T.sz_f), __fmul_rn(d1, T.sz_f)));
-        f2_get(ws, n0, n1);
+        f2_get(rise, n0, n1);
+        n0 = __fadd_rn(n0, __fmul_rn(t0, T.sz_f));
+        n1 = __fadd_rn(n1, __fmul_rn(t1, T.sz_f));
+        const F2 ws = f2(n0, n1);
         f2_get(f2_fma(ws, f2(r.b), one), d0, d1);
         const F2 k = f2(__fdividef(n0, d0), __fdividef(n1, d1));
         cu = f2_mul(k, f2_fma(f2_mul(jf, f2(r.au)), f2(r.b), f2(r.bu)));
@@ -138,7 +142,9 @@ __device__ __forceinline__ void leaf_cost2(const Tile& T, const RayF& r, int32_t
     const F2 top = f2_fma(fu, f2_sub(d10, d00), d00);
     const F2 bot = f2_fma(fu, f2_sub(d11, d01), d01);
     const F2 hb = f2_fma(fv, f2_sub(bot, top), top);
-    const F2 h = kGrid ? rise : f2_add(f2(r.X), rise);
+    float h0, h1;
+    f2_get(rise, h0, h1);
+    const F2 h = kGrid ? rise : f2(__fadd_rn(r.X, h0), __fadd_rn(r.X, h1));
     const F2 it = f2_mul(f2(T.inv_delta_f), f2(rcp_approx(fa), rcp_approx(fb)));
     f2_get(f2_mul(f2_sub(h, hb), it), ca, cb);
 }
