@@ -64,7 +64,7 @@ static __device__ __noinline__ float refine_cost64(const Tile& T, const Rays& R,
 // 81), 38 and 97 us for the Sun and the Earth at 2048^2 (26, 33).
 __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t r,
                                            int32_t bestj, bool stereo, float& light, float& cost) {
-    float uf, vf;
+    float uf, vf, herr = 0.0f;
     DF hp;
     if (R.mode == 0) {
         int32_t u, v;
@@ -77,6 +77,7 @@ __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t
         vf = R.uv[2 * r + 1];
         float href;
         hp = origin_height_df(T, uf, vf, R.lift ? R.lift[r] : 0.0f, href);
+        herr = origin_height_err(T, uf, vf);
     }
     GeomDF F;
     if (stereo)
@@ -85,6 +86,7 @@ __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t
         geom_gnomonic_frame(T, uf, vf, hp, F);
     float err;
     const DF c = leaf_cost_df(T, F, uf, vf, hp, bestj, stereo, err);
+    err += herr / ((float)bestj * T.delta_f);
     // c.hi is the nearest float32 unless c lies within err of the middle between two:
     // half a step of c.hi away from it (a quarter on the inner side of a power of two)
     const uint32_t bits = __float_as_uint(c.hi);
