@@ -65,7 +65,8 @@ struct ViewArgs {
     double step;
     DF dstep;
     float step_f, inv_step;
-    float guard, pos_margin;  // float32 march: heights (m), texel positions
+    float guard;              // float32 march: heights (m)
+    float pos_margin, pos_base, pos_t;   // texel positions (view_margin)
     int64_t K;
     int32_t pool;             // pixels of a march warp
     const float* stats;       // (global max, global min) of the heights
@@ -346,6 +347,11 @@ struct ViewEnd {
     bool ok;
 };
 
+// Bound of the error of a float32 texel position at distance t (see launch_view_rays).
+__device__ __forceinline__ float view_margin(const ViewArgs& a, float t) {
+    return fmaxf(a.pos_margin, fmaf(a.pos_t, t, a.pos_base));
+}
+
 __device__ __forceinline__ ViewEnd view_end(const ViewArgs& a, const ViewRayF& q, float j) {
     ViewEnd e;
     e.t = j * a.step_f;
@@ -361,7 +367,7 @@ __device__ __forceinline__ float view_clear(const ViewArgs& a, const ViewLevels&
                                             const ViewEnd& x, const ViewEnd& y) {
     const Tile& T = a.T;
     const float du = y.u - x.u, dv = y.v - x.v;
-    const float e = a.pos_margin + (du * du + dv * dv) * q.inv8r;
+    const float e = view_margin(a, y.t) + (du * du + dv * dv) * q.inv8r;
     const float lo_u = fminf(x.u, y.u) - e, hi_u = fmaxf(x.u, y.u) + e;
     const float lo_v = fminf(x.v, y.v) - e, hi_v = fmaxf(x.v, y.v) + e;
     const float nxm = (float)(T.nx - 1), nym = (float)(T.ny - 1);
@@ -383,11 +389,12 @@ __device__ __forceinline__ float view_clear(const ViewArgs& a, const ViewLevels&
 __device__ __forceinline__ uint32_t view_leaf(const ViewArgs& a, const ViewRayF& q, uint32_t pix,
                                               uint32_t j0, uint32_t last, float& clear) {
     const Tile& T = a.T;
-    const float nxm = (float)(T.nx - 1), nym = (float)(T.ny - 1), pm = a.pos_margin;
+    const float nxm = (float)(T.nx - 1), nym = (float)(T.ny - 1);
     unsigned hit = 0, doubt = 0;
 #pragma unroll
     for (int i = 0; i < 1 << kViewLeaf; ++i) {
         const ViewEnd e = view_end(a, q, (float)(j0 + i));
+        const float pm = view_margin(a, e.t);
         const bool out = e.ok && (e.u < -pm || e.u > nxm + pm || e.v < -pm || e.v > nym + pm);
         const bool in = e.ok && e.u >= pm && e.u <= nxm - pm && e.v >= pm && e.v <= nym - pm;
         const int32_t i0 = min(max(__float2int_rd(e.u), 0), T.nx - 2);
@@ -950,7 +957,19 @@ cudaError_t launch_view_rays(const Tile& T, const Pyramid& P, const ViewCamera& 
     a.step_f = (float)step;
     a.inv_step = (float)(1.0 / step);
     a.guard = (float)(0.03 + 1e-6 * std::fabs(a.cam.cn - T.R) + 1e-7 * step * (double)K);
+    // Float32 texel positions err by the roundings of the coordinates (1.5e-7 (nx + ny))
+    // and of the point relative to the tile centre's, 2^-24 of its terms, the camera's
+    // distance D0 and tau, times the image's scale (its largest on the tile, heights above
+    // -R/5) and 1 + q for the denominator's.  Replayed against 64-bit mantissas (tiles up to 0.8 radii
+    // wide, cameras 0.1 to 30,000 km up and to 2.5 radii away, texels of 0.2 to 300 m): at
+    // most 1.4 units where the bound takes 4 x 1.25.
+    const double qt = std::hypot((double)(T.nx - 1), (double)(T.ny - 1)) * 0.5 * T.g / T.R;
+    const double scale_max = 1.25 / T.g * (T.proj == 0 ? std::sqrt(1.0 + qt * qt) : 1.0 + 0.25 * qt * qt);
+    const double d0 = std::sqrt(vc.pos[0] * vc.pos[0] + vc.pos[1] * vc.pos[1] +
+                                (vc.pos[2] - T.R) * (vc.pos[2] - T.R));
     a.pos_margin = (float)std::fmax(0.01, 3e-7 * (double)(T.nx + T.ny));
+    a.pos_t = (float)(2.384185791015625e-07 * scale_max * (1.0 + qt));   // 2^-22
+    a.pos_base = (float)(1.5e-7 * (double)(T.nx + T.ny) + (double)a.pos_t * d0);
     a.K = K;
     a.stats = stats;
     const int64_t npix = (int64_t)vc.width * vc.height, nb = view_blocks(vc.width, vc.height);
