@@ -454,13 +454,15 @@ ss_status ss_shade(const ss_heightfield* hf, const ss_rays* rays, const ss_light
  * (h bilinear, decided in FP64); when the sample before it is in the tile too
  * the crossing is refined: bisection of that step until the bracket
  * lies in one bilinear cell, then the single root there of the quadratic that
- * |x| - R - h is along the ray within one cell.  The coordinates lie within one
- * float32 step of the 48-halving FP64 bisection's.  The march runs in float32,
- * samples near the terrain or the tile's border are decided in float-float
- * arithmetic and, where that leaves a doubt, in FP64; the refinement takes
- * float-float values at the two samples and a float32 root between them where
- * its error stays below a quarter of the coordinates' rounding, else FP64
- * (coordinates below 4, tangent rays, steps over several cells).
+ * |x| - R - h is along the ray within one cell, placed within a third of a
+ * float32 step of the texel coordinates (points within 0.25 texel of the tile's
+ * low edges, and near-tangent crossings, bisect on to 2^-36 of the step).  The
+ * march runs in float32; samples near the terrain or the tile's border are
+ * decided in float-float arithmetic and, where that leaves a doubt, in FP64.
+ * The refinement takes float-float values at the two samples and a float32 root
+ * between them, one Newton step in float-float where that root's error could
+ * move the coordinates' rounding, and FP64 where that still could (and for
+ * coordinates below 4, tangent rays, steps over several cells).
  *
  * Output: the hits' texel coordinates (u, v) as float32 pairs in pixel order,
  * uv[2*r], uv[2*r+1] for r < *count (device int64 written by the call), and

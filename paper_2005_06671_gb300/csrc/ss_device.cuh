@@ -579,6 +579,15 @@ __device__ __forceinline__ int32_t df_floor(DF x) {
     return (int32_t)f - ((x.hi == f && x.lo < 0.0f) ? 1 : 0);
 }
 
+// Whether x.hi is the float32 nearest to every value within e of x: unless one lies in the
+// middle between two, half a step of x.hi away from it (a quarter on the inner side of a
+// power of two).
+__device__ __forceinline__ bool df_hi_is_nearest(DF x, float e) {
+    const uint32_t bits = __float_as_uint(x.hi);
+    const float half = __uint_as_float(bits & 0x7f800000u) * 5.9604645e-8f, away = fabsf(x.lo);
+    return away < half - e && ((bits & 0x007fffffu) != 0u || away < 0.5f * half - e);
+}
+
 // Cost of sample j in float-float, (h_p + rise - bilinear height) / t, with heights
 // taken relative to h_p.  err: a bound of its error, 2^-44 of the terms that the sums are
 // made of, whatever cancels in them: sin(eps) (terms up to 1) in the rise, the slopes

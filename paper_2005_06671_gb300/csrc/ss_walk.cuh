@@ -87,13 +87,7 @@ __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t
     float err;
     const DF c = leaf_cost_df(T, F, uf, vf, hp, bestj, stereo, err);
     err += herr / ((float)bestj * T.delta_f);
-    // c.hi is the nearest float32 unless c lies within err of the middle between two:
-    // half a step of c.hi away from it (a quarter on the inner side of a power of two)
-    const uint32_t bits = __float_as_uint(c.hi);
-    const float half = __uint_as_float(bits & 0x7f800000u) * 5.9604645e-8f, away = fabsf(c.lo);
-    cost = c.hi;
-    if (!(away < half - err) || ((bits & 0x007fffffu) == 0u && !(away < 0.5f * half - err)))
-        cost = refine_cost64(T, R, r, bestj, stereo);
+    cost = df_hi_is_nearest(c, err) ? c.hi : refine_cost64(T, R, r, bestj, stereo);
     const float d = cost * sqrtf(fmaxf(0.0f, 1.0f - F.se.hi * F.se.hi)) / T.alpha_f;
     light = disc_light32(d);
 }

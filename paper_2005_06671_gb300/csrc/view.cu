@@ -20,9 +20,9 @@
 // where that leaves a doubt: the first sample found below the terrain is the same
 // one as an FP64 march finds.
 //
-// A second pass gathers each block's hits and refines them with full warps: F at
-// the two samples in float-float, the root between them in float32 relative to
-// those, FP64 where they do not settle it.
+// A second pass gathers the hits and refines them with full warps: F at the two samples
+// in float-float, the root between them in float32 relative to those, one Newton step in
+// float-float where the coordinates' rounding needs it, FP64 where they do not settle it.
 // Then the hits are compacted in pixel order (per-block counts, one scan block,
 // a scatter), so the ray list is deterministic.
 //
@@ -56,6 +56,8 @@ struct Cam {
     // float-float copies: C - P0 (P0 = (0, 0, R)), |C| - R, |C|, |C|^2, |C| + R, R, the image
     // scale, the pixel directions' terms
     DF rel[3], dalt, dcn, dcc, dzsum, dR, dk, df[3], dr[3], du[3], diw, dih;
+    // their error bounds: positions (texels) pos0 + pos_t tau, heights (m) height0 + height_t tau
+    float pos0, pos_t, height0, height_t;
 };
 
 struct ViewArgs {
@@ -75,6 +77,7 @@ struct ViewArgs {
     int32_t* block_count;     // per block of kViewBlock pixels
     int64_t* block_off;       // exclusive prefix of block_count
     int32_t n_blocks;
+    int32_t groups;           // groups of kViewBlock pixels of a refine block
     float* uv_out;
     int32_t* pixel_out;
     int64_t* count_out;
@@ -210,13 +213,16 @@ __device__ __forceinline__ ViewDir view_dir(const Cam& cm, uint32_t pix) {
     return v;
 }
 
-// The point at tau: F = |x| - R - h, its texel image, its bilinear cell, and a
-// bound of F's rounding error.  state: 1 in the tile, 0 off it, -1 in doubt
-// (within the rounding of an edge, or no image).
+// The point at tau: F = |x| - R - h, its texel image, its bilinear cell, and
+// bounds of the rounding errors of F (err) and of the image (pos).  state: 1 in the tile,
+// 0 off it, -1 in doubt (within the rounding of an edge, or no image).
+// The bounds: about 2^-42 of the terms, the distances from the tile centre's point and
+// along the ray among them.  Replayed against 64-bit mantissas (tiles up to 0.8 radii wide,
+// cameras 0.1 to 300,000 km up): at most 0.32 of pos and 0.21 of err used.
 struct ViewPtDF {
     DF f, u, v, rise;
     int32_t i0, j0;
-    float err;
+    float err, pos;
     int state;
 };
 
@@ -240,7 +246,8 @@ __device__ __forceinline__ ViewPtDF view_pt_df(const Tile& T, const Cam& cm, con
     view_image_df(T, cm, r, tau, p.rise, p.u, p.v, den);
     const DF rise = p.rise;
     const float um = (float)(T.nx - 1), vm = (float)(T.ny - 1);
-    const float e = 1e-6f + 1e-11f * (fabsf(p.u.hi) + fabsf(p.v.hi)) + 1e-10f * (um + vm);
+    p.pos = cm.pos0 + cm.pos_t * tau.hi + 2e-14f * (fabsf(p.u.hi) + fabsf(p.v.hi));
+    const float e = 1e-6f + 1e-11f * (fabsf(p.u.hi) + fabsf(p.v.hi)) + 1e-10f * (um + vm) + p.pos;
     const float inside = fminf(fminf(p.u.hi, um - p.u.hi), fminf(p.v.hi, vm - p.v.hi));
     p.f = DF{ 0.0f, 0.0f };
     p.err = 0.0f;
@@ -259,8 +266,8 @@ __device__ __forceinline__ ViewPtDF view_pt_df(const Tile& T, const Cam& cm, con
     const DF hb = df_add(df_mul(fv, df_add(bot, df_neg(top))), top);
     p.f = df_add(df_add(cm.dalt, rise), df_neg(hb));
     const float rng = fmaxf(fmaxf(h00, h10), fmaxf(h01, h11)) - fminf(fminf(h00, h10), fminf(h01, h11));
-    p.err = 1e-12f * (fabsf(cm.dalt.hi) + fabsf(rise.hi) + fabsf(hb.hi)) +
-            1e-12f * (fabsf(p.u.hi) + fabsf(p.v.hi)) * rng;
+    p.err = cm.height0 + cm.height_t * tau.hi + 2e-13f * (fabsf(rise.hi) + fabsf(hb.hi)) +
+            2.0f * p.pos * rng;
     return p;
 }
 
@@ -718,24 +725,35 @@ __device__ __noinline__ float2 view_point64(const ViewArgs& a, uint32_t pix, int
 // image is a line, the rise a parabola and the terrain bilinear cell by cell:
 // F relative to its value at the first point is a quadratic in each cell the step
 // crosses, in float32; the step is halved until both ends lie in one cell (the
-// choices of refine_crossing), whose root is the hit.  False where that does not settle
-// it: a point within rounding of the tile's border or of the terrain, a step of
-// more than one cell line per axis, a tangent ray, a root that the float32
-// coefficients move by more than a quarter of the coordinates' own rounding.
-__device__ __forceinline__ bool view_point_df(const ViewArgs& a, uint32_t pix, int32_t hit_k,
-                                              float2& out) {
+// choices of refine_crossing), whose root is the hit.  The coordinates are the float32
+// nearest to the crossing's: where the error of that root could move their rounding
+// (kViewDoubt: a fifth of the rays at 20 m texels, 1% at 5 m), view_newton takes one step from it.  kViewUnsettled: a
+// point within rounding of the tile's border or of the terrain, a step of more than one cell
+// line per axis, a tangent ray, coordinates below 4.
+// (With roots whose error stayed below a quarter of the rounding instead, 1.8e-3 of the
+// coordinates of 1280 x 720 over 2048^2 of 20 m were one float32 step off; FP64 had 1.7e-5,
+// and so have these.)
+enum { kViewUnsettled, kViewDoubt, kViewDone };
+struct ViewRoot {
+    float s, du, dv, slope, a2, err, off;   // root, image of the step, F there, error bounds
+};
+
+__device__ __forceinline__ int view_point_df(const ViewArgs& a, uint32_t pix, int32_t hit_k,
+                                             float2& out, ViewRoot& root) {
     const Tile& T = a.T;
     const Cam& cm = a.cam;
     const ViewDir r = view_dir(cm, pix);
     const ViewPtDF hi = view_pt_df(T, cm, r, view_tau(a, hit_k));
-    if (hi.state != 1) return false;
+    if (hi.state != 1) return kViewUnsettled;
     out = make_float2(hi.u.hi, hi.v.hi);
-    if (!(fminf(hi.u.hi, hi.v.hi) >= 4.0f)) return false;
-    if (hit_k <= 1) return true;
+    if (!(fminf(hi.u.hi, hi.v.hi) >= 4.0f)) return kViewUnsettled;
+    const int sure = df_hi_is_nearest(hi.u, hi.pos) && df_hi_is_nearest(hi.v, hi.pos) ? kViewDone
+                                                                                      : kViewUnsettled;
+    if (hit_k <= 1) return sure;
     const ViewPtDF lo = view_pt_df(T, cm, r, view_tau(a, hit_k - 1));
-    if (lo.state == 0) return true;     // the sample before the hit is off the tile
-    if (lo.state < 0 || !(lo.f.hi > 4.0f * lo.err) || !(hi.f.hi < -4.0f * hi.err)) return false;
-    if (abs(hi.i0 - lo.i0) > 1 || abs(hi.j0 - lo.j0) > 1) return false;
+    if (lo.state == 0) return sure;     // the sample before the hit is off the tile
+    if (lo.state < 0 || !(lo.f.hi > 4.0f * lo.err) || !(hi.f.hi < -4.0f * hi.err)) return kViewUnsettled;
+    if (abs(hi.i0 - lo.i0) > 1 || abs(hi.j0 - lo.j0) > 1) return kViewUnsettled;
     const float du = df_add(hi.u, df_neg(lo.u)).hi, dv = df_add(hi.v, df_neg(lo.v)).hi;
     const float dr = df_add(hi.rise, df_neg(lo.rise)).hi, h = a.step_f;
     // rise(s) = s dr - K s (1 - s), K = h^2 (1 - (dr/h)^2) / 2 |x|
@@ -772,7 +790,7 @@ __device__ __forceinline__ bool view_point_df(const ViewArgs& a, uint32_t pix, i
         const int32_t mj = min(max((int32_t)floorf(v0 + m * dv), min(bj, fj)), max(bj, fj));
         cell(mi, mj, false);
         const float f = a0 + m * (a1 + m * a2);
-        if (it == 20 || !(fabsf(f) > 1e-6f * (fabsf(lo.f.hi) + relief))) return false;
+        if (it == 20 || !(fabsf(f) > 1e-6f * (fabsf(lo.f.hi) + relief))) return kViewUnsettled;
         if (f > 0.0f) {
             beg = m;
             bi = mi;
@@ -795,46 +813,87 @@ __device__ __forceinline__ bool view_point_df(const ViewArgs& a, uint32_t pix, i
     const float far = fmaxf(fabsf(lo.u.hi - T.cx_f), fabsf(lo.v.hi - T.cy_f));
     const float off = 0.3f * len * hr + 0.5f * far * hr * hr;   // texels
     const float err = 4e-7f * (fabsf(lo.f.hi) + fabsf(dr) + relief) + lo.err + hi.err + K * hr + off * relief;
-    if (!(s >= 0.0f)) return false;
-    const float tol = 1.5e-8f * fabsf(slope) * fminf(lo.u.hi, lo.v.hi);
-    if (err * len + off * fabsf(slope) <= tol) {
-        out = make_float2(df_add(lo.u, DF{ s * du, 0.0f }).hi, df_add(lo.v, DF{ s * dv, 0.0f }).hi);
-    } else {
-        // near the tile's low edges, where float32 steps are short: one Newton step from
-        // F at that root in float-float (p.err is about ten times its error)
-        const ViewPtDF p = view_pt_df(T, cm, r, df_add(view_tau(a, hit_k - 1), df_mul_f(a.dstep, s)));
-        const float ds = -p.f.hi / slope, e = 0.2f * p.err + (fabsf(a2) * ds * ds + 1e-6f * fabsf(ds * slope));
-        if (p.state != 1 || !(fabsf(ds) <= 1e-3f) || !(e * len + off * fabsf(ds * slope) <= tol))
-            return false;
-        out = make_float2(df_add(p.u, DF{ ds * du, 0.0f }).hi, df_add(p.v, DF{ ds * dv, 0.0f }).hi);
-    }
-    return fminf(out.x, out.y) >= 4.0f;
+    if (!(s >= 0.0f)) return kViewUnsettled;
+    // errors of the coordinates: the root's, along the step, the line's, the first point's and
+    // the float32 roundings of s du and s dv
+    const DF u = df_add(lo.u, DF{ s * du, 0.0f }), v = df_add(lo.v, DF{ s * dv, 0.0f });
+    const float e = (__fdividef(err, fabsf(slope)) + 3e-7f) * len + off + lo.pos;
+    out = make_float2(u.hi, v.hi);
+    if (!(fminf(out.x, out.y) >= 4.0f)) return kViewUnsettled;
+    if (df_hi_is_nearest(u, e) && df_hi_is_nearest(v, e)) return kViewDone;
+    root = ViewRoot{ s, du, dv, slope, a2, err, off };
+    return kViewDoubt;
 }
 
-// Pass 2: the hits of a block of pixels, gathered in shared memory so that
-// full warps refine them (a pass-1 warp has a hit in only some of its lanes);
-// writes every pixel's texel coordinates (NaN without a hit) and the block's hit
-// count.
+// One Newton step from a root of view_point_df, from F there in float-float.  False where
+// the rounding of the coordinates is in doubt still.
+__device__ __noinline__ bool view_newton(const ViewArgs& a, uint32_t pix, int32_t hit_k,
+                                            const ViewRoot& q, float2& out) {
+    const ViewDir r = view_dir(a.cam, pix);
+    const ViewPtDF p = view_pt_df(a.T, a.cam, r,
+                                  df_add(view_tau(a, hit_k - 1), df_mul_f(a.dstep, q.s)));
+    const float ds = -p.f.hi / q.slope, rcp = 1.0f / fabsf(q.slope);
+    const DF u = df_add(p.u, DF{ ds * q.du, 0.0f }), v = df_add(p.v, DF{ ds * q.dv, 0.0f });
+    // (the slope is good to what the root's own error and 1e-6 move it)
+    const float es = (p.err + fabsf(ds) * (fabsf(2.0f * q.a2 * ds) + q.err)) * rcp + 1e-6f * fabsf(ds);
+    const float len = fmaxf(fabsf(q.du), fabsf(q.dv));
+    const float e = (es + 2.5e-7f * fabsf(ds)) * len + q.off * fabsf(ds) + p.pos;
+    out = make_float2(u.hi, v.hi);
+    return p.state == 1 && fabsf(ds) <= 1e-3f && df_hi_is_nearest(u, e) && df_hi_is_nearest(v, e) &&
+           fminf(out.x, out.y) >= 4.0f;
+}
+
+// Pass 2: the hits of kViewBlock pixels at a time, gathered in shared memory so that
+// full warps refine them (a pass-1 warp has a hit in only some of its lanes).  Those
+// whose rounding is in doubt wait until a block is full of them, or the last group is
+// done, for view_newton.  Writes every pixel's texel coordinates (NaN without a hit) and
+// the groups' hit counts.
 __global__ void __launch_bounds__(kViewBlock, 4) view_refine_kernel(const __grid_constant__ ViewArgs a) {
     __shared__ int32_t s_pix[kViewBlock];
-    __shared__ int32_t s_cnt;
+    __shared__ uint32_t s_doubt[2 * kViewBlock];
+    __shared__ ViewRoot s_root[2 * kViewBlock];
+    __shared__ int32_t s_cnt, s_cnt2;
     const int64_t npix = (int64_t)a.cam.W * a.cam.H;
-    const int64_t base = (int64_t)blockIdx.x * kViewBlock;
-    const int64_t pix = base + threadIdx.x;
-    if (threadIdx.x == 0) s_cnt = 0;
-    __syncthreads();
-    const bool mine = pix < npix && a.hit_k[pix] >= 0;
-    if (pix < npix && !mine) a.pix_uv[pix] = make_float2(NAN, NAN);
-    if (mine) s_pix[atomicAdd(&s_cnt, 1)] = threadIdx.x;
-    __syncthreads();
-    const int cnt = s_cnt;
-    if (threadIdx.x == 0) a.block_count[blockIdx.x] = cnt;
-    if ((int)threadIdx.x < cnt) {
-        const uint32_t p = (uint32_t)(base + s_pix[threadIdx.x]);
-        const int32_t hit_k = a.hit_k[p];
-        float2 uv;
-        if (!view_point_df(a, p, hit_k, uv)) uv = view_point64(a, p, hit_k);
-        a.pix_uv[p] = uv;
+    const int32_t first = blockIdx.x * a.groups, last = min(first + a.groups, a.n_blocks);
+    if (threadIdx.x == 0) s_cnt2 = 0;
+    for (int32_t g = first; g < last; ++g) {
+        const int64_t base = (int64_t)g * kViewBlock;
+        const int64_t pix = base + threadIdx.x;
+        if (threadIdx.x == 0) s_cnt = 0;
+        __syncthreads();
+        const bool mine = pix < npix && a.hit_k[pix] >= 0;
+        if (pix < npix && !mine) a.pix_uv[pix] = make_float2(NAN, NAN);
+        if (mine) s_pix[atomicAdd(&s_cnt, 1)] = threadIdx.x;
+        __syncthreads();
+        const int cnt = s_cnt;
+        if (threadIdx.x == 0) a.block_count[g] = cnt;
+        if ((int)threadIdx.x < cnt) {
+            const uint32_t p = (uint32_t)(base + s_pix[threadIdx.x]);
+            const int32_t hit_k = a.hit_k[p];
+            float2 uv;
+            ViewRoot root;
+            const int st = view_point_df(a, p, hit_k, uv, root);
+            if (st == kViewDoubt) {
+                const int i = atomicAdd(&s_cnt2, 1);   // (< kViewBlock waited)
+                s_doubt[i] = p;
+                s_root[i] = root;
+            } else {
+                if (st == kViewUnsettled) uv = view_point64(a, p, hit_k);
+                a.pix_uv[p] = uv;
+            }
+        }
+        __syncthreads();
+        const int cnt2 = s_cnt2;
+        if (cnt2 < kViewBlock && g + 1 < last) continue;
+        for (int i = threadIdx.x; i < cnt2; i += kViewBlock) {
+            const uint32_t p = s_doubt[i];
+            const int32_t hit_k = a.hit_k[p];
+            float2 uv;
+            if (!view_newton(a, p, hit_k, s_root[i], uv)) uv = view_point64(a, p, hit_k);
+            a.pix_uv[p] = uv;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_cnt2 = 0;
     }
 }
 
@@ -980,6 +1039,10 @@ cudaError_t launch_view_rays(const Tile& T, const Pyramid& P, const ViewCamera& 
     a.pos_margin = (float)std::fmax(0.01, 3e-7 * (double)(T.nx + T.ny));
     a.pos_t = (float)(2.384185791015625e-07 * scale_max * (1.0 + qt));   // 2^-22
     a.pos_base = (float)(1.5e-7 * (double)(T.nx + T.ny) + (double)a.pos_t * d0);
+    a.cam.pos_t = (float)(2.5e-13 * scale_max * (1.0 + qt));
+    a.cam.pos0 = (float)((double)a.cam.pos_t * d0 + 2e-14 * (double)(T.nx + T.ny));
+    a.cam.height_t = (float)(2e-13 * std::fmax(1.0, 0.5 * a.cam.cn / T.R));
+    a.cam.height0 = (float)(2e-13 * std::fabs(a.cam.cn - T.R) + 4e-16 * a.cam.cn);
     a.K = K;
     a.stats = stats;
     const int64_t npix = (int64_t)vc.width * vc.height, nb = view_blocks(vc.width, vc.height);
@@ -1002,7 +1065,10 @@ cudaError_t launch_view_rays(const Tile& T, const Pyramid& P, const ViewCamera& 
     a.pool = (int32_t)(fill < 32 ? 32 : fill > 256 ? 256 : fill);
     const int64_t per_block = (int64_t)a.pool * (kViewHitBlock / 32);
     view_hit_kernel<<<(unsigned)((npix + per_block - 1) / per_block), kViewHitBlock, 0, s>>>(a);
-    view_refine_kernel<<<(unsigned)nb, kViewBlock, 0, s>>>(a);
+    // groups of a refine block: up to 8 while two waves of resident blocks remain
+    const int64_t groups = nb / ((int64_t)device_sm_count() * 8);
+    a.groups = (int32_t)(groups < 1 ? 1 : groups > 8 ? 8 : groups);
+    view_refine_kernel<<<(unsigned)((nb + a.groups - 1) / a.groups), kViewBlock, 0, s>>>(a);
     view_scan_kernel<<<1, 1024, 0, s>>>(a);
     view_compact_kernel<<<(unsigned)nb, kViewBlock, 0, s>>>(a);
     return cudaGetLastError();
