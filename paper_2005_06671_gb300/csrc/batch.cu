@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(256, SS_BATCH_MIN_BLOCKS) batch_task_kernel(co
             if (done) {
                 const unsigned long long key = TW.key[lane];
                 const int32_t bj = key_j(key);
-                finish_ray(D.T, grid_rays, D.O, L.ray, key_cost(key), bj, nb, nl);
+                finish_ray<false, kRefineCall>(D.T, grid_rays, D.O, L.ray, key_cost(key), bj, nb, nl);
                 if (L.slot >= 0 && bj > 0) {
                     seeds[L.slot] = bj;
                     seed_u[L.slot] = rf.u0;

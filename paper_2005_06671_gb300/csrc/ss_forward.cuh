@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) dp_forward_kernel(cons
             int32_t prev_j = -1;     // a neighbour's argmin, and its origin:
             float su = 0.0f, sv = 0.0f;
             if (done) {
-                finish_ray<kStereo, true>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), w.best, w.bestj,
+                finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), w.best, w.bestj,
                                     w.nb, w.nl);
                 if (colseed && w.bestj > 0) {
                     const int32_t c = seed_col(P, r, LH);
@@ -291,7 +291,7 @@ dp_light_kernel(const __grid_constant__ FwdArgs a) {
         const int n_idle = 32 - __popc(act);
         if (act == 0 || ((open || qn > 0) && n_idle >= a.refill_min)) {
             if (done) {
-                finish_ray<kStereo, true>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), w.best, w.bestj,
+                finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), w.best, w.bestj,
                                           w.nb, w.nl);
                 if (colseed && w.bestj > 0) {
                     const int32_t c = seed_col(P, r, LH);
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel
         unsigned act = __ballot_sync(kFull, r >= 0 && !done);
         if (act == 0 || (open && __popc(~act) >= a.refill_min)) {
             if (done) {
-                finish_ray<kStereo, true>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj, 0, nl);
+                finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj, 0, nl);
                 r = -1;
                 done = false;
             }
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel
                                            0.5f * rf.B * rf.B * rf.inv_2rho);
                     G = 3.0f * kGuardRel * (rf.guard0 + fabsf(hmax_rel) + rb);
                     if (rf.j_hi < rf.j_lo) {   // no usable sample: written at once
-                        finish_ray<kStereo, true>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj,
+                        finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj,
                                                   0, 0);
                         r = -1;
                     }

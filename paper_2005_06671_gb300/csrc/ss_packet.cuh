@@ -640,7 +640,7 @@ __device__ __forceinline__ void pk_packet(const Tile& T, const LevelTab& L, int3
     const unsigned long long key = W.key[lane];
     const int32_t bj = kLight && key_j(key) == 0 ? -1 : key_j(key);
     if (live)
-        finish_ray<kStereo, true>(T, R, O, ray, key_cost(key), bj, kCount ? W.cnt[0][lane] : 0,
+        finish_ray<kStereo, kRefineLater>(T, R, O, ray, key_cost(key), bj, kCount ? W.cnt[0][lane] : 0,
                                   kCount ? W.cnt[1][lane] : 0);
     prev_j = bj;
     pu = u0;

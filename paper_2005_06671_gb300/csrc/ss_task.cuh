@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) dp_task_kernel(const F
             if (done) {
                 const unsigned long long key = W.key[lane];
                 const int32_t bj = key_j(key);
-                finish_ray<kStereo, true>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), key_cost(key),
+                finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), key_cost(key),
                                           bj, nb, nl);
                 if (bj > 0) {
                     const int32_t c = seed_col(P, r, LH);

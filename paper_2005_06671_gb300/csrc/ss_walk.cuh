@@ -92,15 +92,40 @@ __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t
     light = disc_light32(d);
 }
 
+// The same in FP64, for walks that re-evaluate in their services, a lane or two of a warp
+// at a time: there float-float's instructions and registers cost more than FP64's
+// latency.  Batch of four tiles of 300^2 to 1024^2, FP64 inlined / called / float-float
+// inlined: light-only 913 / 930 / 967 us, sun 30 to 50 degrees 961 / 962 / 1085; leaves as
+// tasks 11.6 / 10.9 / 11.2 ms.
+__device__ __forceinline__ void refine_ray64(const Tile& T, const Rays& R, int64_t r,
+                                             int32_t bestj, bool stereo, float& light, float& cost) {
+    double up, vp, hp, href, ow[4];
+    int32_t oi0, oj0;
+    ray_origin(T, R, r, up, vp, hp, href, oi0, oj0, ow);
+    Geom64 G;
+    geom64_any(T, up, vp, hp, G, stereo);
+    const double c = leaf_cost64(T, G, bestj, stereo);
+    const float se = (float)G.sin_e;
+    light = disc_light32((float)c * sqrtf(fmaxf(0.0f, 1.0f - se * se)) / T.alpha_f);
+    cost = (float)c;
+}
+
+static __device__ __noinline__ void refine_ray64_call(const Tile& T, const Rays& R, int64_t r,
+                                                     int32_t bestj, bool stereo, float& light,
+                                                     float& cost) {
+    refine_ray64(T, R, r, bestj, stereo, light, cost);
+}
+
 // Light value marking a ray whose re-evaluation is left to refine_kernel.
 constexpr float kLightPending = -1.0f;
 
-// Final value of one ray: the float-float re-evaluation of its argmin sample unless
+// Final value of one ray: the FP64 re-evaluation of its argmin sample unless
 // the light is certainly saturated (|c*| cos(eps) >= 1.001 alpha), then the
-// disc-occlusion formula (Eq. discfrac).  kDefer: leave the re-evaluation to
-// refine_kernel (light = kLightPending), so that the walk's warp services
-// carry no re-evaluation with a lane or two active.
-template <bool kStereo = false, bool kDefer = false>
+// disc-occlusion formula (Eq. discfrac).  kRefine: in FP64 here, inlined or called, or
+// left to refine_kernel (refine_ray; light = kLightPending), so that the walk's warp
+// services carry no re-evaluation with a lane or two active.
+enum { kRefineHere, kRefineLater, kRefineCall };
+template <bool kStereo = false, int kRefine = kRefineHere>
 __device__ __forceinline__ void finish_ray(const Tile& T, const Rays& R, const Outputs& O,
                                            int64_t r, float best, int32_t bestj, int32_t nb,
                                            int32_t nl) {
@@ -112,12 +137,15 @@ __device__ __forceinline__ void finish_ray(const Tile& T, const Rays& R, const O
     } else if (fabsf(best) * cos_elev_f32(T, R, r, kStereo) >= 1.001f * T.alpha_f) {
         light = best > 0.0f ? 1.0f : 0.0f;
         cost = best;
-    } else if (kDefer) {
+    } else if (kRefine == kRefineLater) {
         light = kLightPending;
         cost = 0.0f;
         write_cost = false;
     } else {
-        refine_ray(T, R, r, bestj, kStereo, light, cost);
+        if (kRefine == kRefineCall)
+            refine_ray64_call(T, R, r, bestj, kStereo, light, cost);
+        else
+            refine_ray64(T, R, r, bestj, kStereo, light, cost);
     }
     O.light[r] = light;
     O.argmin[r] = bestj;
