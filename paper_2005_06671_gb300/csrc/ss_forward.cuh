@@ -365,6 +365,15 @@ dp_light_kernel(const __grid_constant__ FwdArgs a) {
     }
 }
 
+// Re-evaluation of a ray left pending.
+template <bool kStereo>
+__device__ __forceinline__ void refine_pending(const FwdArgs& a, int64_t r) {
+    float light, cost;
+    refine_ray(a.T, a.R, r, a.O.argmin[r], kStereo, light, cost);
+    a.O.light[r] = light;
+    if (a.O.cost) a.O.cost[r] = cost;
+}
+
 // ---------------------------------------------------------------- uniform
 // Every usable sample in order, same scheduling as the descent.  Early exit
 // (exact): with H(t) = h_p + rise(t) convex and H(0) = h_p <= max h,
@@ -374,7 +383,8 @@ dp_light_kernel(const __grid_constant__ FwdArgs a) {
 // Penumbra rays are left to refine_kernel: float-float inside the services, with a lane
 // or two active and more registers, took 27.3 ms exact / 9.5 ms light-only at 2048^2 and
 // 32.7 / 12.3 ms on a stereographic tile (FP64 there: 26.4 / 9.0, 29.8 / 11.4; now 25.6 /
-// 8.8, 29.4 / 11.2).
+// 8.8, 29.4 / 11.2).  Small launches (kUniOwnRefine) re-evaluate their block's rays at its
+// end instead of a second launch: 2^2 to 16^2 3 us less (29 -> 26, stereographic 79 -> 76).
 template <bool kCount, bool kGrid, bool kPoly, bool kLight, bool kStereo>
 __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel(const FwdArgs a) {
     __shared__ int32_t s_next;
@@ -394,7 +404,8 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel
         unsigned act = __ballot_sync(kFull, r >= 0 && !done);
         if (act == 0 || (open && __popc(~act) >= a.refill_min)) {
             if (done) {
-                finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj, 0, nl);
+                finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj,
+                                                  0, nl);
                 r = -1;
                 done = false;
             }
@@ -414,8 +425,8 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel
                                            0.5f * rf.B * rf.B * rf.inv_2rho);
                     G = 3.0f * kGuardRel * (rf.guard0 + fabsf(hmax_rel) + rb);
                     if (rf.j_hi < rf.j_lo) {   // no usable sample: written at once
-                        finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r), best, bestj,
-                                                  0, 0);
+                        finish_ray<kStereo, kRefineLater>(a.T, a.R, a.O, chunk_ray(P, a.T.nx, r),
+                                                          best, bestj, 0, 0);
                         r = -1;
                     }
                 }
@@ -441,6 +452,13 @@ __global__ void __launch_bounds__(256, SS_FWD_MIN_BLOCKS) uniform_forward_kernel
         }
         ++j;
         done = kLight ? (stop || best <= -rf.c_sat) : stop;
+    }
+    if (a.own_refine) {
+        __syncthreads();
+        for (int32_t i = threadIdx.x; i < P.cnt; i += blockDim.x) {
+            const int64_t id = chunk_ray(P, a.T.nx, i);
+            if (a.O.light[id] == kLightPending) refine_pending<kStereo>(a, id);
+        }
     }
 }
 
@@ -472,11 +490,7 @@ __global__ void __launch_bounds__(256) refine_kernel(const FwdArgs a, int rounds
     __syncthreads();
     const int cnt = s_cnt;
     for (int i = threadIdx.x; i < cnt; i += 256) {
-        const int64_t r = s_ray[i];
-        float light, cost;
-        refine_ray(a.T, a.R, r, a.O.argmin[r], kStereo, light, cost);
-        a.O.light[r] = light;
-        if (a.O.cost) a.O.cost[r] = cost;
+        refine_pending<kStereo>(a, s_ray[i]);
     }
 }
 
@@ -549,11 +563,15 @@ struct DpLaunch {
     }
 };
 
+constexpr int64_t kUniOwnRefine = 1024;   // rays
+
 template <bool C, bool G, bool P, bool L, bool S>
 struct UniLaunch {
     static cudaError_t go(const FwdArgs& a, int grid, int block, cudaStream_t s) {
-        uniform_forward_kernel<C, G, P, L, S><<<grid, block, 0, s>>>(a);
-        launch_refine<S>(a, s);
+        FwdArgs b = a;
+        b.own_refine = (a.R.mode == 0 ? (int64_t)a.T.nx * a.T.ny : a.R.n) <= kUniOwnRefine;
+        uniform_forward_kernel<C, G, P, L, S><<<grid, block, 0, s>>>(b);
+        if (!b.own_refine) launch_refine<S>(a, s);
         return cudaGetLastError();
     }
 };

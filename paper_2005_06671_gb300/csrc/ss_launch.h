@@ -51,6 +51,7 @@ struct FwdArgs {
     int32_t colseed;          // descent, grid rays in rectangles: column seeds
     int32_t seed_w;           // descent: half-width of a seed window
     PkShape pk;               // packet descent
+    int32_t own_refine;       // uniform stepping: blocks re-evaluate their own rays
 };
 
 constexpr int32_t kColSeedMaxW = 512;    // widest rectangle with a column-seed table
