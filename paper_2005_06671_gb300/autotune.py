@@ -1,8 +1,8 @@
 """Autotuner for the batched forward's launch shape.
 
-Searches, by coordinate descent from the library's default (packets of 32 rays,
-every field 0 or -1), over the shapes of the single-ray walks, which any field set
-selects:
+Times the library's default (packets of rays, every field 0 or -1), then searches by
+coordinate descent over the shapes of the single-ray walks, which any field set selects,
+from their own best in sweeps, and returns the fastest of all:
   block_threads   threads per block
   rays_per_thread rays per warp = 32 x this (one queue chunk)
   ray_tile_w      chunk shape: 0 = runs of consecutive texels, w = w x (rays/w) rectangles
@@ -33,10 +33,17 @@ SPACE = {
     "leaf_level": (-1, 1, 2, 3),
     "strip_len": (0, 1, 6, 10, 16),
 }
-# the starting point: the library's own choice, packets of rays (16 tiles of 512^2 to
-# 4096^2 on GB300: 32.6 ms against 89.9 ms for the walks in 64 x 64 chunks, their own best in sweeps)
+# the library's own choice, packets of rays (16 tiles of 512^2 to 4096^2 on GB300: 32.6 ms
+# against 89.9 ms for WALK)
 DEFAULT = {"block_threads": 0, "rays_per_thread": 0, "ray_tile_w": 0, "refill_min": 0,
            "leaf_level": -1, "strip_len": 0}
+# where the descent over the walks starts: 64 x 64 chunks, services at 14 idle lanes, leaf
+# blocks of 4 samples as warp tasks.  (From DEFAULT it could not leave: every step is a
+# walk with the other fields at their defaults, slower than the packets it left.)
+WALK = {"block_threads": 256, "rays_per_thread": 128, "ray_tile_w": 64, "refill_min": 14,
+        "leaf_level": 1, "strip_len": 0}
+# fields whose 0 (-1) is a walk's default under another name
+SAME_AS_WALK = ("block_threads", "rays_per_thread", "refill_min", "leaf_level")
 
 
 def default_table_path():
@@ -82,8 +89,9 @@ def time_batch(hfs, suns, max_len_m, params, reps=3, step_texels=0.5):
 
 
 def tune(hfs, suns, max_len_m, reps=3, rounds=2, step_texels=0.5, log=None):
-    """Coordinate descent over SPACE; returns (best params, {key: ms})."""
-    best = dict(DEFAULT)
+    """DEFAULT, or the walk that coordinate descent over SPACE finds, whichever is faster;
+    returns (best params, {key: ms})."""
+    best = dict(WALK)
     seen = {}
 
     def cost(p):
@@ -94,6 +102,7 @@ def tune(hfs, suns, max_len_m, reps=3, rounds=2, step_texels=0.5, log=None):
                 log(f"autotune {key} {seen[key]:.3f} ms")
         return seen[key]
 
+    packets_ms = cost(dict(DEFAULT))
     best_ms = cost(best)
     for _ in range(rounds):
         improved = False
@@ -102,12 +111,14 @@ def tune(hfs, suns, max_len_m, reps=3, rounds=2, step_texels=0.5, log=None):
                 cand = dict(best, **{name: v})
                 if cand == best or not _valid(cand):
                     continue
+                if name in SAME_AS_WALK and v == DEFAULT[name]:
+                    continue
                 ms = cost(cand)
                 if ms < best_ms:
                     best, best_ms, improved = cand, ms, True
         if not improved:
             break
-    return best, seen
+    return (dict(DEFAULT) if packets_ms <= best_ms else best), seen
 
 
 def load_table(path=None):
