@@ -1309,11 +1309,11 @@ __device__ __forceinline__ float probe(const Tile& T, const LevelTab& L, int32_t
         const float dx = xb - xa, dy = yb - ya;
         e += (dx * dx + dy * dy) * r.inv8r;
     }
-    // clamped before the +1, so no conversion result can overflow
-    int32_t x0 = max(__float2int_rd(fminf(xa, xb) - e), 0);
-    int32_t x1 = min(__float2int_rd(fmaxf(xa, xb) + e), T.nx - 2) + 1;
-    int32_t y0 = max(__float2int_rd(fminf(ya, yb) - e), 0);
-    int32_t y1 = min(__float2int_rd(fmaxf(ya, yb) + e), T.ny - 2) + 1;
+    // clamped both ways, and before the +1: a box off the tile reads cells of its border
+    int32_t x0 = __vimin_s32_relu(__float2int_rd(fminf(xa, xb) - e), T.nx - 1);
+    int32_t x1 = __vimin_s32_relu(__float2int_rd(fmaxf(xa, xb) + e), T.nx - 2) + 1;
+    int32_t y0 = __vimin_s32_relu(__float2int_rd(fminf(ya, yb) - e), T.ny - 1);
+    int32_t y1 = __vimin_s32_relu(__float2int_rd(fmaxf(ya, yb) + e), T.ny - 2) + 1;
     const int32_t ext = max(x1 - x0, y1 - y0);
     int32_t m = ext <= 1 ? 0 : 31 - __clz(ext);
     m += (((x1 >> m) - (x0 >> m)) > 1 || ((y1 >> m) - (y0 >> m)) > 1) ? 1 : 0;

@@ -130,10 +130,11 @@ __device__ __forceinline__ float block_bound(const Tile& T, const LevelTab& L, i
         const float dx = xb - xa, dy = yb - ya;
         e += (dx * dx + dy * dy) * r.inv8r;
     }
-    const int32_t x0 = max(__float2int_rd(fminf(xa, xb) - e), 0);
-    const int32_t x1 = min(__float2int_rd(fmaxf(xa, xb) + e), T.nx - 2) + 1;
-    const int32_t y0 = max(__float2int_rd(fminf(ya, yb) - e), 0);
-    const int32_t y1 = min(__float2int_rd(fmaxf(ya, yb) + e), T.ny - 2) + 1;
+    // (clamped both ways: a box off the tile reads cells of its border)
+    const int32_t x0 = __vimin_s32_relu(__float2int_rd(fminf(xa, xb) - e), T.nx - 1);
+    const int32_t x1 = __vimin_s32_relu(__float2int_rd(fmaxf(xa, xb) + e), T.nx - 2) + 1;
+    const int32_t y0 = __vimin_s32_relu(__float2int_rd(fminf(ya, yb) - e), T.ny - 1);
+    const int32_t y1 = __vimin_s32_relu(__float2int_rd(fmaxf(ya, yb) + e), T.ny - 2) + 1;
     const int32_t ext = max(x1 - x0, y1 - y0);
     int32_t m = ext <= 1 ? 0 : 31 - __clz(ext);
     m += (((x1 >> m) - (x0 >> m)) > 1 || ((y1 >> m) - (y0 >> m)) > 1) ? 1 : 0;
