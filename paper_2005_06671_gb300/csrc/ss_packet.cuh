@@ -297,7 +297,7 @@ __device__ __forceinline__ void pk_leaf_pass(const Tile& T, Warp& W, PkRings& Q,
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             j[i] = min(j0 + i * d, jh);
-            if (!kGrid) j[i] = max(j[i], jl);   // (a grid ray's first usable sample is 1)
+            if (!kGrid || kStereo) j[i] = max(j[i], jl);
         }
 #pragma unroll
         for (int i = 0; i < 4; i += 2) {
@@ -328,6 +328,9 @@ __device__ __forceinline__ void pk_leaf_pass(const Tile& T, Warp& W, PkRings& Q,
 template <bool kCount, bool kGrid, bool kPoly, bool kLight, bool kStereo, class Warp>
 __device__ __forceinline__ void pk_node_pass(const Tile& T, const LevelTab& L, int32_t levels,
                                              Warp& W, PkRings& Q, int lane) {
+    // a gnomonic grid ray's usable samples start at 1.  (A stereographic one's image is an
+    // arc: from a texel on the tile's border it can bulge out and come in again.)
+    constexpr bool kFirst = kGrid && !kStereo;
     const int n = kGrid || Q.nc <= kPkStackFull ? min(32, Q.nc) : 8;
     bool pa = false, pb = false;
     int32_t s = 0, k = kPkNodeLog;
@@ -349,10 +352,13 @@ __device__ __forceinline__ void pk_node_pass(const Tile& T, const LevelTab& L, i
         const float best = key_cost(W.key[slot]);
         if (kLight && best <= -W.csat[slot]) jh = 0;   // in full umbra: nothing more to find
         const int32_t half = kGrid ? kPkNode / 2 : 1 << (k - 1);
-        // (ends clipped to the last usable sample: past it the image may leave the plane,
-        // 1 + b j <= 0, and a box to there would miss the samples)
+        // (ends clipped to the usable samples: beyond them the image may leave the plane,
+        // 1 + b j <= 0, or pass the antipode, and a box to there would miss the samples)
         const float fs = (float)s, fh = (float)half, fj = (float)jh;
-        const float j0 = fs + 1.0f, j1 = fminf(fs + (fh + 0.5f), fj), j2 = fminf(fs + 2.0f * fh, fj);
+        const float fl = kFirst ? 1.0f : (float)jl;
+        const float j0 = kFirst ? fs + 1.0f : fmaxf(fs + 1.0f, fl);
+        const float j1 = fmaxf(fminf(fs + (fh + 0.5f), fj), fl);
+        const float j2 = fmaxf(fminf(fs + 2.0f * fh, fj), fl);
         const float t0 = j0 * T.delta_f, t1 = j1 * T.delta_f, t2 = j2 * T.delta_f;
         float x0, y0, x1, y1, x2, y2;
         block_end<kStereo>(T, r, j0, t0, kStereo ? rise_of<kPoly>(r, t0) : 0.0f, x0, y0);
@@ -371,8 +377,8 @@ __device__ __forceinline__ void pk_node_pass(const Tile& T, const LevelTab& L, i
         const float hg = __fmaf_rn(-0.2503f * q.y * dt, dt, q.w);
         const float f0 = pk_f(q.y, p, hg, t0), f1 = pk_f(q.y, p, hg, t1);
         const float f2 = pk_f(q.y, p, hg, t2);
-        pa = !(fminf(f0, f1) > Ma) && s + 1 <= jh && (kGrid || s + half >= jl);
-        pb = !(fminf(f1, f2) > Mb) && s + half + 1 <= jh && (kGrid || s + 2 * half >= jl);
+        pa = !(fminf(f0, f1) > Ma) && s + 1 <= jh && (kFirst || s + half >= jl);
+        pb = !(fminf(f1, f2) > Mb) && s + half + 1 <= jh && (kFirst || s + 2 * half >= jl);
         if (kCount) atomicAdd(&W.cnt[0][slot], 2);
     }
     if (kGrid) Q.nh = (Q.nh + n) & (kPkNodeRing - 1);
