@@ -1163,6 +1163,15 @@ __device__ __forceinline__ float leaf_cost(const Tile& T, const RayF& r, int32_t
     return __fmul_rn(__fsub_rn(h, hb), inv_t(T, jf));
 }
 
+// How far an arc of at most half the image circle bulges from its chord: the sagitta
+// r - sqrt(r^2 - L^2/4) is at most (L^2 / 8r) (1 + L^2 / 4r^2).  (Without the second factor it
+// is short by L^2/16r^2 of itself: texels where a block of 256 samples is a radian.)
+// l2: L^2, inv8r: 1 / 8r.
+__device__ __forceinline__ float arc_bulge(float l2, float inv8r) {
+    const float a = l2 * inv8r;
+    return fmaf(16.0f * a * inv8r, a, a);
+}
+
 // float32 texel position of sample j for block footprints (error <= pos_eps);
 // rise = rise(t_j) (used by the stereographic mapping only)
 template <bool kStereo>
@@ -1307,7 +1316,7 @@ __device__ __forceinline__ float probe(const Tile& T, const LevelTab& L, int32_t
     float e = r.pos_eps;
     if (kStereo) {
         const float dx = xb - xa, dy = yb - ya;
-        e += (dx * dx + dy * dy) * r.inv8r;
+        e += arc_bulge(dx * dx + dy * dy, r.inv8r);
     }
     // clamped both ways, and before the +1: a box off the tile reads cells of its border
     int32_t x0 = __vimin_s32_relu(__float2int_rd(fminf(xa, xb) - e), T.nx - 1);

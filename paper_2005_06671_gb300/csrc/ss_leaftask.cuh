@@ -128,7 +128,7 @@ __device__ __forceinline__ float block_bound(const Tile& T, const LevelTab& L, i
     float e = r.pos_eps;
     if (kStereo) {   // the arc bulges from its chord by at most its sagitta
         const float dx = xb - xa, dy = yb - ya;
-        e += (dx * dx + dy * dy) * r.inv8r;
+        e += arc_bulge(dx * dx + dy * dy, r.inv8r);
     }
     // (clamped both ways: a box off the tile reads cells of its border)
     const int32_t x0 = __vimin_s32_relu(__float2int_rd(fminf(xa, xb) - e), T.nx - 1);

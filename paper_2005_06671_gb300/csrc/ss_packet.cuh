@@ -266,7 +266,7 @@ __device__ __forceinline__ float pk_union_max(const Tile& T, const LevelTab& L, 
             yhi = fmaxf(yhi, U.v0[1] + fmaxf(nvh * il, nvh * ih));
         }
         const float dx = xhi - xlo, dy = yhi - ylo;
-        e += (dx * dx + dy * dy) * U.inv8r;
+        e += arc_bulge(dx * dx + dy * dy, U.inv8r);
     }
     // (a NaN or an overflow in the ranges prunes nothing)
     if (!(xhi - xlo < 1e7f && yhi - ylo < 1e7f)) return INFINITY;
@@ -366,8 +366,8 @@ __device__ __forceinline__ void pk_node_pass(const Tile& T, const LevelTab& L, i
         block_end<kStereo>(T, r, j2, t2, kStereo ? rise_of<kPoly>(r, t2) : 0.0f, x2, y2);
         float ea = q.x, eb = q.x;
         if (kStereo) {
-            ea += ((x1 - x0) * (x1 - x0) + (y1 - y0) * (y1 - y0)) * r.inv8r;
-            eb += ((x2 - x1) * (x2 - x1) + (y2 - y1) * (y2 - y1)) * r.inv8r;
+            ea += arc_bulge((x1 - x0) * (x1 - x0) + (y1 - y0) * (y1 - y0), r.inv8r);
+            eb += arc_bulge((x2 - x1) * (x2 - x1) + (y2 - y1) * (y2 - y1), r.inv8r);
         }
         const float Ma = pk_box_max(T, L, levels, fminf(x0, x1) - ea, fmaxf(x0, x1) + ea,
                                     fminf(y0, y1) - ea, fmaxf(y0, y1) + ea);

@@ -379,7 +379,7 @@ __device__ __forceinline__ float view_clear(const ViewArgs& a, const ViewLevels&
                                             const ViewEnd& x, const ViewEnd& y) {
     const Tile& T = a.T;
     const float du = y.u - x.u, dv = y.v - x.v;
-    const float e = view_margin(a, y.t) + (du * du + dv * dv) * q.inv8r;
+    const float e = view_margin(a, y.t) + arc_bulge(du * du + dv * dv, q.inv8r);
     const float lo_u = fminf(x.u, y.u) - e, hi_u = fmaxf(x.u, y.u) + e;
     const float lo_v = fminf(x.v, y.v) - e, hi_v = fmaxf(x.v, y.v) + e;
     const float nxm = (float)(T.nx - 1), nym = (float)(T.ny - 1);

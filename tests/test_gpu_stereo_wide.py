@@ -43,3 +43,13 @@ def _same(R, g, n, elev, az, shapes=(dict(), dict(block_threads=256))):
     (2e3, 5.0, 300, 25.0, 351.4), (2e3, 66.6, 84, 2.0, 200.0), (2e3, 20.0, 90, 25.0, 351.4)])
 def test_rays_that_start_off_the_tile(R, g, n, elev, az):
     _same(R, g, n, elev, az)
+
+
+# Tiles of up to the whole hemisphere of a small body: blocks of samples whose images are arcs
+# of up to a radian and more.
+@pytest.mark.parametrize("R,g,n", [(2e3, 66.6, 84), (2e3, 40.0, 140), (2e3, 20.0, 280),
+                                   (2e3, 5.0, 500), (1e5, 250.0, 1000)])
+@pytest.mark.parametrize("elev,az", [(2.0, 351.4), (25.0, 49.0), (-20.0, 300.0)])
+def test_tiles_of_a_hemisphere(R, g, n, elev, az):
+    assert 0.5 * math.hypot(n - 1, n - 1) * g <= 2.0 * R
+    _same(R, g, n, elev, az)
