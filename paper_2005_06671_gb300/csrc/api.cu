@@ -151,6 +151,8 @@ ss::Tile make_tile(const ss_heightfield* hf, const ss_sun* sun, int32_t J, doubl
     split(s[1], sy_hi, T.sy_lo);
     split(2.0 * R / g, T.k2_hi, T.k2_lo);
     split(s[2] / R, T.szR_f, T.szR_lo);
+    T.beyond = hf->projection != SS_PROJ_GNOMONIC && hypot(T.cx, T.cy) * g > 1.9999 * R;
+    T.pos_base = 1e-3f + 5e-7f * (float)(T.nx + T.ny) + (T.beyond ? 2.0f * (T.nx + T.ny) : 0.0f);
     return T;
 }
 

@@ -62,6 +62,13 @@ struct Tile {
     float Rsx_hi, Rsx_lo, Rsy_hi, Rsy_lo, sz_lo, szR_f, szR_lo;
     // and for the stereographic setup: sx, sy (low words), 2R/g
     float sx_lo, sy_lo, k2_hi, k2_lo;
+    // Footprint margin (texels) but for the terms of a ray: 1e-3 + 5e-7 (nx + ny), more
+    // than the tile where `beyond` is set: stereographic tiles that reach beyond the
+    // hemisphere around the pole (corner distance > 2R).  Within it the image of a ray
+    // between two samples is the shorter arc of its circle; beyond it can be the longer one,
+    // through the surroundings of the antipode, which no box of its ends covers.
+    float pos_base;
+    int32_t beyond;
 };
 
 struct Rays {
@@ -766,7 +773,7 @@ __device__ __forceinline__ void make_rayf_gnomonic_grid(const Tile& T, int32_t u
         sample_range(T, G, r.j_lo, r.j_hi);
     }
     const float amax = fmaxf(fabsf(r.au), fabsf(r.av));
-    r.pos_eps = 1e-3f + 5e-7f * (float)(T.nx + T.ny) + 8e-7f * amax * (float)max(r.j_hi, 1);
+    r.pos_eps = T.pos_base + 8e-7f * amax * (float)max(r.j_hi, 1);
     set_gconst(T, r);
 }
 
@@ -827,7 +834,7 @@ __device__ __forceinline__ void make_rayf_gnomonic(const Tile& T, double up, dou
         sample_range(T, G, r.j_lo, r.j_hi);
     }
     const float amax = fmaxf(fabsf(r.au), fabsf(r.av));
-    r.pos_eps = 1e-3f + 5e-7f * (float)(T.nx + T.ny) + 8e-7f * amax * (float)max(r.j_hi, 1);
+    r.pos_eps = T.pos_base + 8e-7f * amax * (float)max(r.j_hi, 1);
     set_gconst(T, r);
 }
 
@@ -1003,7 +1010,7 @@ __device__ __forceinline__ void make_rayf(const Tile& T, const Geom64& G, double
         r.inv8r = (float)(G.nz_cross * T.g / (16.0 * T.R));
         r.au = __fadd_rn(r.au_hi, r.au_lo);
         r.av = __fadd_rn(r.av_hi, r.av_lo);
-        if (!sample_range_stereo_f32(T, G, r, r.j_lo, r.j_hi))
+        if (T.beyond || !sample_range_stereo_f32(T, G, r, r.j_lo, r.j_hi))
             sample_range_stereo(T, G, r.j_lo, r.j_hi);
 #ifdef SS_RANGE_CHECK
         {   // test builds: the float32 search against the FP64 one
@@ -1021,7 +1028,7 @@ __device__ __forceinline__ void make_rayf(const Tile& T, const Geom64& G, double
     // float32 block-end positions u0 + a*tau err by <= ulp(coordinate) plus
     // ~3 ulp of a*tau; the margin takes 4x that, plus 1e-3 texel
     float amax = fmaxf(fabsf((float)G.Au), fabsf((float)G.Av));
-    r.pos_eps = 1e-3f + 5e-7f * (float)(T.nx + T.ny) + 8e-7f * amax * (float)max(r.j_hi, 1);
+    r.pos_eps = T.pos_base + 8e-7f * amax * (float)max(r.j_hi, 1);
     if (kStereo) {
         // the stereographic end positions also carry w * B with |w| <= 2 t
         const float bmax = fmaxf(fabsf(r.bu), fabsf(r.bv));
@@ -1198,7 +1205,8 @@ __device__ __forceinline__ void block_end(const Tile& T, const RayF& r, float jf
 //    outside; E is the walk's footprint margin taken at j = J (a bound of the
 //    float32 position error over the whole ray) plus the rounding of the
 //    margin itself;
-//  * the ray's image is a circle arc of radius rc = 1/(8 inv8r) texels, and the
+//  * the ray's image is a circle arc of radius rc = 1/(8 inv8r) texels, at most half the
+//    circle (the tile does not reach beyond the hemisphere), and the
 //    samples between two samples lie on the arc between them, within
 //    L^2/(4 rc) of its chord (length L, L < rc); the chord is as far inside
 //    the tile as its nearer end, so when both ends are inside by more than

@@ -53,3 +53,12 @@ def test_rays_that_start_off_the_tile(R, g, n, elev, az):
 def test_tiles_of_a_hemisphere(R, g, n, elev, az):
     assert 0.5 * math.hypot(n - 1, n - 1) * g <= 2.0 * R
     _same(R, g, n, elev, az)
+
+
+# Tiles that reach beyond the hemisphere: a ray's image between two samples on the tile can
+# be the arc of its circle that passes the antipode, far off the tile.
+@pytest.mark.parametrize("R,g,n", [(2e3, 20.0, 700), (2e3, 66.7, 90), (5e3, 60.0, 301)])
+@pytest.mark.parametrize("elev,az", [(2.0, 171.9), (25.0, 49.0), (-20.0, 300.0)])
+def test_tiles_beyond_the_hemisphere(R, g, n, elev, az):
+    assert 0.5 * math.hypot(n - 1, n - 1) * g > 2.0 * R
+    _same(R, g, n, elev, az, shapes=(dict(), dict(block_threads=256), dict(lane_leaves=True)))
