@@ -100,8 +100,9 @@ enum { SS_RAYS_GRID = 0, SS_RAYS_LIST = 1 };
  * bound reaches it cannot change the light) and stops as soon as
  * best <= -c_sat (the ray is in full umbra).  light is exact as in the default
  * mode; argmin and cost are exact for rays in the penumbra; a fully lit ray
- * reports argmin -1, cost +inf; a ray in umbra reports the first sample found
- * with cost <= -c_sat (a witness, not necessarily the minimum). */
+ * reports argmin -1, cost +inf; a ray in umbra reports a sample with cost
+ * <= -c_sat (a witness, not necessarily the minimum: which one depends on the
+ * order of the search, and so on the launch shape). */
 #define SS_FLAG_LIGHT_ONLY 0x4u
 
 /* ss_shadow_backward_ws: deterministic accumulation (see there). */
@@ -141,8 +142,11 @@ typedef struct {
     double angular_radius_rad;  /* alpha = r_L > 0                             */
 } ss_sun;
 
-/* The descent (ss_shadow_forward, the batch) takes packets of 32 rays when every
- * shape field below is left at its default (and SS_FLAG_LANE_LEAVES is not set).
+/* The descent (ss_shadow_forward, the batch) takes packets of neighbouring rays (32,
+ * or 16 or 8 for launches that would leave warps free) when every shape field below
+ * is left at its default (and SS_FLAG_LANE_LEAVES is not set), rays are at most 2.5e5
+ * texels long, and the items of a batch take the same form of the rise (the series
+ * for short rays and low suns, else the closed form).
  * Setting any of block_threads, leaf_level, rays_per_thread, refill_min,
  * ray_tile_w, strip_len or seed_width selects the single-ray walks, where the
  * fields left at 0 (-1) take the defaults given with them.  Same results. */
@@ -323,7 +327,7 @@ ss_status ss_shadow_backward_ws(const ss_heightfield* hf, const ss_rays* rays, c
  * counterpart in the paper is drawing many visible tiles per frame (Sec. 3.3,
  * virtual texturing; Sec. 6.3).  Grid-mode rays (one per texel centre),
  * gnomonic tiles.  params (max_len_m, step_texels, ...) apply to every item;
- * default shape fields select packets of 32 rays, strips of which are the queue's
+ * default shape fields select packets of rays, strips of which are the queue's
  * chunks; with a shape field set the rest take the walks' batch defaults: exact
  * walks in 64 x 64 chunks of texels (rays_per_thread 128, ray_tile_w 64) with column seeds and services
  * at 14 idle lanes, light-only walks in runs of 512 (rays_per_thread 16) with

@@ -8,8 +8,8 @@
 // instance is ever in flight in the warp.  Penumbra rays are left pending and
 // re-evaluated by a second kernel over the same strips, with full warps.
 //
-// Bound by instruction issue, as ss_packet.cuh.  16 tiles of 512^2 to 4096^2 (67 M
-// rays, a sun each) take 33.6 ms against 89.9 ms with batch_task_kernel; 16 tiles of
+// Bound by instruction issue, as ss_packet.cuh.  16 tiles of 512^2 to 4096^2 (89 M
+// rays, a sun each) take 32.6 ms against 89.9 ms with batch_task_kernel; 16 tiles of
 // 512^2 1.69 against 11.7 ms, 4 tiles of 256^2 0.17 against 7.3 ms (its chunks of
 // 4,096 texels leave most of the GPU's warps without one).
 #include "ss_batch.h"
