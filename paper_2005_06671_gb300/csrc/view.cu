@@ -28,8 +28,9 @@
 //
 // What bounds it: the FP64 pipe (77% / 86% busy, GB300 runs it at 1/64 of the float32
 // rate) while setup, doubtful samples and refinement were FP64; now instruction
-// issue (72% in the march, 17 of 32 lanes: rays differ in length).  3840 x 2160 over
-// 16384^2, 6.2 M hits: 18.55 -> 4.12 ms; 1920 x 1080 over 8192^2 4.83 -> 1.34 ms;
+// issue in the march (75% of slots, 21 of 32 lanes: rays differ in length), and in the
+// refinement the few hits that FP64 settles (issue 31%, FP64 pipe 61%, waits at barriers).  3840 x 2160 over
+// 16384^2, 6.2 M hits: 18.55 -> 4.22 ms; 1920 x 1080 over 8192^2 4.83 -> 1.37 ms;
 // 640 x 360 over 2048^2 of 20 m 1.26 -> 0.40 ms.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -732,7 +733,7 @@ __device__ __noinline__ float2 view_point64(const ViewArgs& a, uint32_t pix, int
 // line per axis, a tangent ray, coordinates below 4.
 // (With roots whose error stayed below a quarter of the rounding instead, 1.8e-3 of the
 // coordinates of 1280 x 720 over 2048^2 of 20 m were one float32 step off; FP64 had 1.7e-5,
-// and so have these.)
+// these have 1.7e-6.)
 enum { kViewUnsettled, kViewDoubt, kViewDone };
 struct ViewRoot {
     float s, du, dv, slope, a2, err, off;   // root, image of the step, F there, error bounds
@@ -825,10 +826,11 @@ __device__ __forceinline__ int view_point_df(const ViewArgs& a, uint32_t pix, in
     return kViewDoubt;
 }
 
-// One Newton step from a root of view_point_df, from F there in float-float.  False where
-// the rounding of the coordinates is in doubt still.
-__device__ __noinline__ bool view_newton(const ViewArgs& a, uint32_t pix, int32_t hit_k,
-                                            const ViewRoot& q, float2& out) {
+// One Newton step from a root of view_point_df, from F there in float-float.  Where the
+// rounding of the coordinates is in doubt still, one more from F in FP64 (good to its
+// rounding, 2e-9 m, over the slope: what refine_crossing takes seven values of F for).
+__device__ __noinline__ float2 view_newton(const ViewArgs& a, uint32_t pix, int32_t hit_k,
+                                           const ViewRoot& q) {
     const ViewDir r = view_dir(a.cam, pix);
     const ViewPtDF p = view_pt_df(a.T, a.cam, r,
                                   df_add(view_tau(a, hit_k - 1), df_mul_f(a.dstep, q.s)));
@@ -838,15 +840,23 @@ __device__ __noinline__ bool view_newton(const ViewArgs& a, uint32_t pix, int32_
     const float es = (p.err + fabsf(ds) * (fabsf(2.0f * q.a2 * ds) + q.err)) * rcp + 1e-6f * fabsf(ds);
     const float len = fmaxf(fabsf(q.du), fabsf(q.dv));
     const float e = (es + 2.5e-7f * fabsf(ds)) * len + q.off * fabsf(ds) + p.pos;
-    out = make_float2(u.hi, v.hi);
-    return p.state == 1 && fabsf(ds) <= 1e-3f && df_hi_is_nearest(u, e) && df_hi_is_nearest(v, e) &&
-           fminf(out.x, out.y) >= 4.0f;
+    if (p.state != 1 || !(fabsf(ds) <= 1e-3f) || !(fminf(u.hi, v.hi) >= 4.0f))
+        return view_point64(a, pix, hit_k);
+    if (df_hi_is_nearest(u, e) && df_hi_is_nearest(v, e)) return make_float2(u.hi, v.hi);
+    double d[3];
+    pixel_dir(a.cam, pix, d);
+    const double tau = ((double)(hit_k - 1) + ((double)q.s + (double)ds)) * a.step;
+    const ViewPt w = view_pt(a.T, a.cam.C, d, tau);
+    const double dw = -w.f / (double)q.slope;
+    if (!w.in || !(fabs(dw) <= 1e-6)) return view_point64(a, pix, hit_k);
+    return make_float2((float)(w.u + dw * (double)q.du), (float)(w.v + dw * (double)q.dv));
 }
 
 // Pass 2: the hits of kViewBlock pixels at a time, gathered in shared memory so that
 // full warps refine them (a pass-1 warp has a hit in only some of its lanes).  Those
 // whose rounding is in doubt wait until a block is full of them, or the last group is
-// done, for view_newton.  Writes every pixel's texel coordinates (NaN without a hit) and
+// done, for view_newton.  (3840 x 2160: 4.22 ms; one group per block 4.33; hits left to FP64
+// waiting as well 4.34.)  Writes every pixel's texel coordinates (NaN without a hit) and
 // the groups' hit counts.
 __global__ void __launch_bounds__(kViewBlock, 4) view_refine_kernel(const __grid_constant__ ViewArgs a) {
     __shared__ int32_t s_pix[kViewBlock];
@@ -887,10 +897,7 @@ __global__ void __launch_bounds__(kViewBlock, 4) view_refine_kernel(const __grid
         if (cnt2 < kViewBlock && g + 1 < last) continue;
         for (int i = threadIdx.x; i < cnt2; i += kViewBlock) {
             const uint32_t p = s_doubt[i];
-            const int32_t hit_k = a.hit_k[p];
-            float2 uv;
-            if (!view_newton(a, p, hit_k, s_root[i], uv)) uv = view_point64(a, p, hit_k);
-            a.pix_uv[p] = uv;
+            a.pix_uv[p] = view_newton(a, p, a.hit_k[p], s_root[i]);
         }
         __syncthreads();
         if (threadIdx.x == 0) s_cnt2 = 0;
