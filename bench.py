@@ -38,10 +38,10 @@ CONFIG = "mid"
 # One launch of the descent kernel on the 4096x4096 workload, from one ncu capture
 # (profiles/dp_task_grid4096.md; None until taken for the current kernel):
 # dram__bytes_read.sum + dram__bytes_write.sum, and the issue counters
-MID_DP_TRAFFIC_BYTES = 91290112 + 101828864
-MID_DP_ISSUE = {"smsp__inst_executed.sum": 6007537388,
-                "smsp__thread_inst_executed.sum": 181693707185,
-                "sm__cycles_elapsed.avg": 13416470.58, "gpu__time_duration.sum_ns": 6488928}
+MID_DP_TRAFFIC_BYTES = 90744320 + 101957120
+MID_DP_ISSUE = {"smsp__inst_executed.sum": 6059758593,
+                "smsp__thread_inst_executed.sum": 183308867673,
+                "sm__cycles_elapsed.avg": 13848709.24, "gpu__time_duration.sum_ns": 6694048}
 SMS, SMSP_PER_SM = 152, 4
 DESCENT_KERNEL = "dp_packet_kernel"
 

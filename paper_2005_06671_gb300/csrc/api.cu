@@ -285,10 +285,11 @@ ss_status shadow_common(FwdKind kind, const ss_heightfield* hf, const float* mip
                    : descent              ? 10
                                           : 6;
     // Packets of rays (ss_packet.cuh) unless a launch shape is asked for: faster than
-    // the walks for every size, mapping, ray set and mode measured, from 1.2x
-    // (2048^2, light-only, sun 0.3 deg: 1.31 -> 1.06 ms) over 2.2x (4096^2: 15.9 -> 7.1 ms)
-    // to 15x (100 k scattered points: 3.3 -> 0.22 ms); the same within 5 us below
-    // 1,500 rays.  The walks stay for callers that set a shape.
+    // the walks for every size, mapping, ray set and mode measured, from 1.4x
+    // (2048^2 stereographic, light-only, sun 75 deg: 2.61 -> 1.91 ms) over 2.2x (4096^2: 15.3
+    // -> 6.8 ms) to 17x (100 k scattered points: 3.2 -> 0.19 ms) and more for small tiles
+    // (256^2: 1.31 -> 0.055 ms); one listed ray 37 -> 28 us.  The walks stay for callers that
+    // set a shape.
     if (descent && takes_packets(params, J))
         a.pk = ss::pk_shape(rays->mode == SS_RAYS_GRID
                                 ? ss::pk_grid_strips(hf->nx, hf->ny, ss::PkShape{ 32, 1 })

@@ -30,16 +30,16 @@
 // ray down (pk_descend_list); the rest is the same.
 //
 // What bounds it: instruction issue (76% of slots at 2048^2, 30 of 32 lanes active,
-// the ALU pipe 51% busy, shared and L1 wavefronts 63%, DRAM 0.1%); per packet of 32
-// rays 11.4 k instructions: 12 leaf passes 3.8 k, 13 node passes ~3 k, tests 1 k,
+// the ALU pipe 52% busy, shared and L1 wavefronts 65%, DRAM 0.1%); per packet of 32
+// rays 11.5 k instructions: 12 leaf passes 3.8 k, 13 node passes ~3 k, tests 1 k,
 // setup 0.6 k, unions 0.4 k.  Measured (GB300, pass with the mipmap) against the task
-// descent of ss_task.cuh: 4096^2 15.9 -> 7.1 ms, 1531 x 1021 2.71 -> 0.74 ms, 256^2
-// 1.15 -> 0.076 ms, 1200 x 1000 stereographic 3.83 -> 0.87 ms, 1.04 M view points
-// 13.2 -> 1.9 ms, 100 k scattered points 3.5 -> 0.21 ms (the task descent's
+// descent of ss_task.cuh: 4096^2 15.3 -> 6.8 ms, 1531 x 1021 2.49 -> 0.72 ms, 256^2
+// 1.15 -> 0.063 ms, 1200 x 1000 stereographic 3.59 -> 0.84 ms, 1.04 M view points
+// 9.8 -> 1.9 ms, 100 k scattered points 3.2 -> 0.19 ms (the task descent's
 // blocks of 6,144 or 3,072 rays leave most SMs idle on all but the first).
 // Scalar leaves, tests and one push per node of the packet took 8.0 ms at 4096^2;
-// tasks of 16 samples bounded in quarters 7.0, but light-only passes 9% and view
-// points 16% more.
+// tasks of 16 samples bounded in quarters 7.0 (against 7.1 then), but light-only passes
+// 9% and view points 16% more.
 #pragma once
 
 #include "ss_forward.cuh"

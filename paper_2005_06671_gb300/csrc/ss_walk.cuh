@@ -60,8 +60,8 @@ static __device__ __noinline__ float refine_cost64(const Tile& T, const Rays& R,
 // cost to FP64's float32, the disc formula (Eq. discfrac) in float32 (error < 1e-7 in
 // light).  The cost is taken in float-float; where its error could move the
 // rounding to float32 (two rays in a thousand), in FP64.  All in FP64, ~180
-// operations at 1/64 of the float32 rate, refine_kernel took 133 us at 4096^2 (now
-// 81), 38 and 97 us for the Sun and the Earth at 2048^2 (26, 33).
+// operations at 1/64 of the float32 rate, refine_kernel took 133 us at 4096^2 (now 98), 64
+// us on average for the Sun and the Earth at 2048^2 (29).
 __device__ __forceinline__ void refine_ray(const Tile& T, const Rays& R, int64_t r,
                                            int32_t bestj, bool stereo, float& light, float& cost) {
     float uf, vf, herr = 0.0f;
